@@ -9,15 +9,10 @@
 // scattered 16-byte pieces; the quad then sums its partial contractions with
 // two shuffles.  Flexible replicas keep positions, velocities and forces in
 // shared memory; the integrator updates run with lanes over atoms.
-#include <math.h>
-
+#include <type_traits>
 #include <vector>
 
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
-#include "internal.h"
-#include "interp.cuh"
+#include "replica_common.cuh"
 
 namespace {
 
@@ -27,21 +22,6 @@ constexpr int kThreads = 32 * kWarpsPerBlock;
 #define GRIDFF_MIN_BLOCKS_PER_SM 4
 #endif
 constexpr int kMinBlocksPerSM = GRIDFF_MIN_BLOCKS_PER_SM;
-constexpr int kQuads = 8;                 // atoms evaluated per warp at a time
-constexpr int kMaxA = GRIDFF_MAX_ATOMS;
-constexpr unsigned kFull = 0xffffffffu;
-
-struct FireP {
-  float dt_start, dt_max, f_inc, f_dec, alpha_start, f_alpha, d_max, f_conv2;
-  int n_min;
-};
-
-struct Control {
-  const volatile int* abort_flag;   // host-mapped
-  unsigned long long budget_ns;     // 0 = none
-  DevResult* res;
-};
-
 // per-warp shared state of a flexible replica
 struct WarpState {
   float x[3 * kMaxA];
@@ -57,184 +37,15 @@ struct WarpStateXF {
   float x[3 * kMaxA];
   float f[3 * kMaxA];
 };
-__device__ __forceinline__ void store_eg(WarpState& s, int i, float e) { s.eg[i] = e; }
-__device__ __forceinline__ void store_eg(WarpStateXF&, int, float) {}
-
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ float wsum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-__device__ __forceinline__ double wsum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-__device__ __forceinline__ float qsum(float v) {
-  v += __shfl_xor_sync(kFull, v, 1);
-  v += __shfl_xor_sync(kFull, v, 2);
-  return v;
-}
-
-// Per-warp stencil cache in shared memory.  Slot i (i < S) holds, for the
-// atom evaluated by a quad, the 64 node values c = Q b^C + P b^P + L b^L
-// of its 4x4x4 stencil (combined with that atom's fixed factors) and the
-// cell they belong to.  Between consecutive steps an atom usually stays in
-// its cell, so the gather is served from shared memory; it goes to global
-// memory only when the cell changes.  Layout: lane q of the quad holds the
-// 16 values of node z+q-1 for the 16 (x, y) runs, as 4 float4; float4 j of
-// lane q of slot i sits at index (j * S + i) * 4 + q, so a warp access to 8
-// consecutive slots is contiguous (no bank conflicts).
-struct StencilCache {
-  float4* val;   // [4 * S * 4]
-  int* key;      // [S] packed cell index, -1 = empty
-  int S;
+// per-warp shared state of an evaluation
+struct WarpStateEval {
+  float x[3 * kMaxA];
+  float f[3 * kMaxA];
+  float eg[kMaxA];
 };
-
-// Channel-combined values c = Q C + P P + L L of the 16 (x, y) runs at one
-// z-node: records base + a sx + b nzp, run m = 4a + b, for the grid's record
-// kind (channel scales folded into the atom's factors; the branch is
-// uniform over the warp).
-// KIND >= 0: the record kind is known at compile time (no other code is
-// generated); KIND < 0: dispatch on g.kind.
-template <int KIND = -1>
-__device__ __forceinline__ void gather_runs(const GridView& g, long long base, float4 par, float cv[16]) {
-  const float fc = par.x * g.sC, fp = par.y * g.sP, fl = par.z * g.sL;
-  switch (KIND >= 0 ? KIND : g.kind) {
-    case REC_F32x4: {
-      const float4* p = (const float4*)g.rec + base;
-      float4 r[16];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) r[m] = __ldg(p + (m >> 2) * g.sx + (m & 3) * g.nzp);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) cv[m] = fmaf(fc, r[m].x, fmaf(fp, r[m].y, fl * r[m].z));
-      break;
-    }
-    case REC_F32x2: {
-      const float2* p = (const float2*)g.rec + base;
-      float2 r[16];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) r[m] = __ldg(p + (m >> 2) * g.sx + (m & 3) * g.nzp);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) cv[m] = fmaf(fp, r[m].x, fl * r[m].y);
-      break;
-    }
-    case REC_F16x4:
-    case REC_BF16x4: {
-      const uint2* p = (const uint2*)g.rec + base;
-      uint2 r[16];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) r[m] = __ldg(p + (m >> 2) * g.sx + (m & 3) * g.nzp);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        float2 a, b;
-        if (g.kind == REC_F16x4) {
-          a = __half22float2(*reinterpret_cast<const __half2*>(&r[m].x));
-          b = __half22float2(*reinterpret_cast<const __half2*>(&r[m].y));
-        } else {
-          a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[m].x));
-          b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[m].y));
-        }
-        cv[m] = fmaf(fc, a.x, fmaf(fp, a.y, fl * b.x));
-      }
-      break;
-    }
-    default: {   // REC_F16x2, REC_BF16x2
-      const unsigned* p = (const unsigned*)g.rec + base;
-      unsigned r[16];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) r[m] = __ldg(p + (m >> 2) * g.sx + (m & 3) * g.nzp);
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        const float2 a = g.kind == REC_F16x2 ? __half22float2(*reinterpret_cast<const __half2*>(&r[m]))
-                                             : __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r[m]));
-        cv[m] = fmaf(fp, a.x, fl * a.y);
-      }
-      break;
-    }
-  }
-}
-
-// Energy and force of one atom in the substrate field (Eqs. E, E_Coulomb,
-// E_Morse), evaluated by the 4 lanes of a quad (q = lane & 3); every lane of
-// the quad returns the full result.  Lane q gathers record q of each of
-// the 16 z-runs (one warp load fetches 8 whole 64-byte runs), combines the
-// channels with the atom's factors (Q, P, L), accumulates the x/y-weighted
-// sums for node z+q-1, applies its own z weight, and the quad sums.  The
-// force is minus the analytic gradient of the interpolant (Sec. 5).
-// `act` false: the quad has no atom (it still takes part in the shuffles).
-// `slot` >= 0: the atom may use stencil-cache slot `slot`.
-// kPartial: return this lane's share (the 4 shares of a quad sum to the
-// atom's value) instead of the quad sum.
-template <bool kPartial = false, int KIND = -1>
-__device__ __forceinline__ void grid_quad(const GridView& g, int q, bool act, float x, float y, float z,
-                                          float4 par, float& e, float& fx, float& fy, float& fz, int& flags,
-                                          const StencilCache& sc, int slot) {
-  const Cell cl = locate(g, act, x, y, z, flags);
-  float wx[4], dwx[4], wy[4], dwy[4], wz[4], dwz[4];
-  bspline_weights(cl.tx, wx, dwx);
-  bspline_weights(cl.ty, wy, dwy);
-  bspline_weights(cl.tz, wz, dwz);
-  float cv[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) cv[j] = 0.f;
-  if (cl.inside) {
-    const int key = (cl.ix * g.ny + cl.iy) * g.nz + cl.iz;
-    const bool cached = slot >= 0 && slot < sc.S;
-    if (cached && sc.key[slot] == key) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float4 v = sc.val[(j * sc.S + slot) * 4 + q];
-        cv[4 * j] = v.x;
-        cv[4 * j + 1] = v.y;
-        cv[4 * j + 2] = v.z;
-        cv[4 * j + 3] = v.w;
-      }
-    } else {
-      gather_runs<KIND>(g, ((long long)cl.ix * g.nyp + cl.iy) * g.nzp + cl.iz + q, par, cv);
-      if (cached) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          sc.val[(j * sc.S + slot) * 4 + q] = make_float4(cv[4 * j], cv[4 * j + 1], cv[4 * j + 2], cv[4 * j + 3]);
-        if (q == 0) sc.key[slot] = key;
-      }
-    }
-  }
-  float S0 = 0.f, Sx = 0.f, Sy = 0.f;
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    float s = 0.f, sy = 0.f;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      s = fmaf(wy[b], cv[4 * a + b], s);
-      sy = fmaf(dwy[b], cv[4 * a + b], sy);
-    }
-    S0 = fmaf(wx[a], s, S0);
-    Sx = fmaf(dwx[a], s, Sx);
-    Sy = fmaf(wx[a], sy, Sy);
-  }
-  const float wq = q == 0 ? wz[0] : q == 1 ? wz[1] : q == 2 ? wz[2] : wz[3];
-  const float dwq = q == 0 ? dwz[0] : q == 1 ? dwz[1] : q == 2 ? dwz[2] : dwz[3];
-  e = wq * S0;
-  fx = -wq * Sx * g.inv_dx;
-  fy = -wq * Sy * g.inv_dy;
-  fz = -dwq * S0 * g.inv_dz;
-  if (!kPartial) {
-    e = qsum(e);
-    fx = qsum(fx);
-    fy = qsum(fy);
-    fz = qsum(fz);
-  }
-}
-
-// Bytes of one warp's cache with S slots (a multiple of 16).
-__host__ __device__ constexpr size_t cache_bytes(int S) { return (size_t)S * 256 + (((size_t)S * 4 + 15) & ~size_t(15)); }
+__device__ __forceinline__ void store_eg(WarpState& s, int i, float e) { s.eg[i] = e; }
+__device__ __forceinline__ void store_eg(WarpStateEval& s, int i, float e) { s.eg[i] = e; }
+__device__ __forceinline__ void store_eg(WarpStateXF&, int, float) {}
 
 // Bytes of one replica's share in the sub-warp kernels: its stencil cache
 // and the cells its lanes publish for the refill queue (int2 per slot).
@@ -257,27 +68,6 @@ __device__ __forceinline__ StencilCache warp_cache(unsigned char* dyn, int S, in
 __device__ __forceinline__ void cache_reset(const StencilCache& sc, int lane) {
   for (int i = lane; i < sc.S; i += 32) sc.key[i] = -1;
   __syncwarp();
-}
-
-__device__ __forceinline__ float3 ld3(const float* s, int i) {
-  return make_float3(s[3 * i], s[3 * i + 1], s[3 * i + 2]);
-}
-__device__ __forceinline__ float3 sub3(float3 a, float3 b) { return make_float3(a.x - b.x, a.y - b.y, a.z - b.z); }
-__device__ __forceinline__ float dot3(float3 a, float3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-__device__ __forceinline__ float3 cross3(float3 a, float3 b) {
-  return make_float3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
-}
-
-// cos(n phi) and sin(n phi) from cos phi and sin phi by n rotations in the
-// complex plane (exact trigonometry, no angle): (c, s) <- (c, s) e^{i phi}.
-__device__ __forceinline__ void multiple_angle(float cphi, float sphi, int n, float& cn, float& sn) {
-  cn = 1.f;
-  sn = 0.f;
-  for (int k = 0; k < n; ++k) {
-    const float c2 = fmaf(cn, cphi, -sn * sphi);
-    sn = fmaf(sn, cphi, cn * sphi);
-    cn = c2;
-  }
 }
 
 // This lane's share (terms q, q+4, ... of each list; partners q, q+4, ...)
@@ -404,10 +194,6 @@ __device__ __forceinline__ void quat_advance(float q[4], float ux, float uy, flo
   q[3] = z * inv;
 }
 
-__device__ __forceinline__ bool finite3(float a, float b, float c) {
-  return isfinite(a) && isfinite(b) && isfinite(c);
-}
-
 // Per-replica stop check (abort flag, clock budget), every 32 steps.
 __device__ __forceinline__ int stop_bits(const Control& ctl, unsigned long long t0, int lane) {
   int bits = 0;
@@ -416,14 +202,6 @@ __device__ __forceinline__ int stop_bits(const Control& ctl, unsigned long long 
     if (ctl.budget_ns && gtimer() - t0 > ctl.budget_ns) bits |= GRIDFF_REP_STEPLIMIT;
   }
   return __shfl_sync(kFull, bits, 0);
-}
-
-__device__ __forceinline__ void report(const Control& ctl, int n, int evals, int st, int steps) {
-  atomicAdd(&ctl.res->atom_evals, (unsigned long long)n * (unsigned long long)evals);
-  if (st & GRIDFF_REP_CONVERGED) atomicAdd(&ctl.res->n_converged, 1);
-  atomicMax(&ctl.res->max_steps, steps);
-  int sb = st & (GRIDFF_REP_ABORTED | GRIDFF_REP_STEPLIMIT);
-  if (sb) atomicOr(&ctl.res->stop_bits, sb);
 }
 
 // Record of a replica's final evaluation (the one after which a relaxation
@@ -501,18 +279,6 @@ __device__ __forceinline__ Acc flex_forces(const GridView& g, bool use_grid, boo
 // lane's share of the energy.  Same terms as
 // intra_quad (reduced UFF-like form; nonbonded on pairs more than two bonds
 // apart), without the per-atom repetition.
-__device__ __forceinline__ uint32_t pick4(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, int k) {
-  return k == 0 ? w0 : k == 1 ? w1 : k == 2 ? w2 : w3;
-}
-
-// 2^x by the PTX instruction ex2.approx.ftz.f32 (relative error about 2^-22).
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-constexpr float kLog2e = 1.44269504088896341f;   // log2(e)
-
 // Nonbonded force factor c (F_i = c d, d = x_i - x_j) and energy of one pair
 // (Morse with mixed R_i + R_j and eps_i eps_j, plus Coulomb), from per-atom
 // factors prepared once per replica: pi = {k_e q_i, a R_i, eps_i, -} for
@@ -585,8 +351,9 @@ __device__ __forceinline__ float3 nb_steps(const float* s_x, const float4* s_nb,
   return g;
 }
 
-__device__ float intra_terms(const TemplateView& tv, int t, int lane, const float* s_x, float* s_f,
-                             const float4* s_nb) {
+template <class Acc>
+__device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float* s_x, float* s_f, const float4* s_nb) {
+  Acc enb = Acc(0);
   float e = 0.f;
   const float alpha = tv.alpha;
   const int n = tv.natoms[t], ab = tv.atom_off[t];
@@ -646,6 +413,10 @@ __device__ float intra_terms(const TemplateView& tv, int t, int lane, const floa
       s_f[3 * i + 1] += fi.y;
       s_f[3 * i + 2] += fi.z;
     }
+    if (sizeof(Acc) > sizeof(float)) {   // FP64 energies: FP32 sums over one block's partners at most
+      enb += (Acc)e;
+      e = 0.f;
+    }
   }
   __syncwarp();
   // Bonded terms (few per atom): lanes take terms round-robin and add the
@@ -704,7 +475,7 @@ __device__ float intra_terms(const TemplateView& tv, int t, int lane, const floa
     sh_add3(s_f, T.d, m3 * B.x, m3 * B.y, m3 * B.z);
     e += 0.5f * T.V * (1.f - T.cn0 * cn);
   }
-  return e;
+  return enb + (Acc)e;
 }
 
 // Forces of one flexible replica (positions in s.x) with the grid term by
@@ -742,7 +513,7 @@ __device__ __forceinline__ Acc flex_forces_terms(const GridView& g, bool use_gri
     }
   }
   __syncwarp();
-  if (use_intra) e += (Acc)intra_terms(tv, t, lane, s.x, s.f, s_nb);
+  if (use_intra) e += intra_terms<Acc>(tv, t, lane, s.x, s.f, s_nb);
   __syncwarp();
   return e;
 }
@@ -797,17 +568,20 @@ __device__ __forceinline__ void rigid_forces(const GridView& g, const TemplateVi
 // ---------------------------------------------------------------------------
 // evaluation (no update)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, kMinBlocksPerSM)
+__global__ void __launch_bounds__(kThreads, 2 * kMinBlocksPerSM)
 eval_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
-            const int* __restrict__ rep_off, int n_rep, int rigid, const float* __restrict__ xs,
+            const int* __restrict__ rep_off, const int* __restrict__ order, int n_rep, int rigid, const float* __restrict__ xs,
             int use_grid, int use_intra, double* __restrict__ E_out, float* __restrict__ F_out,
             float* __restrict__ Ea_out, int* __restrict__ st_out) {
-  __shared__ WarpState s_all[kWarpsPerBlock];
+  __shared__ WarpStateEval s_all[kWarpsPerBlock];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  WarpState& s = s_all[wib];
+  __shared__ float4 s_nb_all[kWarpsPerBlock][kMaxA];
+  WarpStateEval& s = s_all[wib];
+  float4* const s_nb = s_nb_all[wib];
   const int warp = blockIdx.x * kWarpsPerBlock + wib;
   const int n_warps = gridDim.x * kWarpsPerBlock;
-  for (int r = warp; r < n_rep; r += n_warps) {
+  for (int k = warp; k < n_rep; k += n_warps) {   // largest molecules first
+    const int r = order[k];
     const int t = rep_tmpl[r], n = tv.natoms[t], ab = tv.atom_off[t], off = rep_off[r];
     __syncwarp();
     if (rigid) {
@@ -821,11 +595,17 @@ eval_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
         s.x[3 * i + 2] = Rm[6] * b.x + Rm[7] * b.y + Rm[8] * b.z + p[2];
       }
     } else {
-      for (int k = lane; k < 3 * n; k += 32) s.x[k] = xs[3 * (size_t)off + k];
+      for (int m = lane; m < 3 * n; m += 32) s.x[m] = xs[3 * (size_t)off + m];
+      for (int i = lane; i < n; i += 32) {
+        float4 p = __ldg(&tv.nb[ab + i]);
+        p.y *= tv.alpha * kLog2e;
+        s_nb[i] = p;
+      }
+      pad_pair_slots(s.x, s_nb, n, lane);
     }
     int flags = 0;
     const StencilCache nocache{nullptr, nullptr, 0};
-    double E = flex_forces(g, use_grid, use_intra && !rigid, tv, ab, n, lane, s, flags, nocache);
+    double E = flex_forces_terms<double>(g, use_grid, use_intra && !rigid, tv, t, ab, n, lane, s, flags, nocache, s_nb);
     for (int i = lane; i < n; i += 32) {
       float* f = F_out + 3 * ((size_t)off + i);
       f[0] = s.f[3 * i];
@@ -1752,8 +1532,9 @@ relax_flex_terms_kernel(GridView g, TemplateView tv, const int* __restrict__ rep
 }
 
 // ---------------------------------------------------------------------------
-// Langevin dynamics of flexible replicas (the thermalisation of minima
-// hopping, Sec. 7), BAOAB splitting: half kick, half drift, exact
+// Dynamics of flexible replicas.  NVE: velocity Verlet, the potential energy
+// accumulated in FP64 per lane, total energies recorded every rec_every steps.
+// Langevin (the thermalisation of minima hopping, Sec. 7), BAOAB splitting: half kick, half drift, exact
 // Ornstein-Uhlenbeck velocity update v <- c1 v + c2 sqrt(kT/m) xi, half
 // drift, forces, half kick; c1 = exp(-gamma dt), c2 = sqrt(1 - c1^2).
 // xi of replica r, global step s, component m = 3 i + a:
@@ -1761,13 +1542,14 @@ relax_flex_terms_kernel(GridView g, TemplateView tv, const int* __restrict__ rep
 // Layout as relax_flex_terms_kernel (warp per replica, work queue, GC: the
 // global stencil cache).
 // ---------------------------------------------------------------------------
-template <int WPB, int KIND, bool GC>
+template <int WPB, int KIND, bool GC, bool NVE>
 __global__ void __launch_bounds__(32 * WPB, GRIDFF_FLEX_WARPS_PER_SM / WPB)
-langevin_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
+md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
                      const int* __restrict__ rep_off, const int* __restrict__ order, int n_rep, float* xs,
                      float* vs, int* status, double* energy, int nsteps, float dt, float c1, float c2,
-                     float kT_acc, unsigned long long seed, long long step0, Control ctl, int use_grid,
-                     int use_intra, int S, float4* gval, int* gkey) {
+                     float kT_acc, unsigned long long seed, long long step0, int rec_every, double* trace,
+                     int trace_stride, Control ctl, int use_grid, int use_intra, int S, float4* gval, int* gkey) {
+  using Acc = typename std::conditional<NVE, double, float>::type;
   __shared__ WarpState s_all[WPB];
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1804,25 +1586,57 @@ langevin_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tm
       s.x[m] = xs[3 * (size_t)off + m];
       s.v[m] = vs[3 * (size_t)off + m];
     }
-    // nonbonded factors {q, alpha log2(e) R, eps} and 1/sqrt(m) in the
+    // nonbonded factors {q, alpha log2(e) R, eps} and 1/m or 1/sqrt(m) in the
     // free fourth slot; zeros up to the next multiple of 32 atoms
     for (int i = lane; i < n; i += 32) {
       float4 p = __ldg(&tv.nb[ab + i]);
       p.y *= tv.alpha * kLog2e;
-      p.w = rsqrtf(__ldg(&tv.body[ab + i]).w);
+      const float mass = __ldg(&tv.body[ab + i]).w;
+      p.w = NVE ? 1.f / mass : rsqrtf(mass);
       s_nb[i] = p;
     }
     pad_pair_slots(s.x, s_nb, n, lane);
-    int st = status[r] & ~(GRIDFF_REP_CONVERGED | GRIDFF_REP_ABORTED | GRIDFF_REP_STEPLIMIT);
+    int st = status[r] & ~((NVE ? 0 : GRIDFF_REP_CONVERGED) | GRIDFF_REP_ABORTED | GRIDFF_REP_STEPLIMIT);
     int flags = 0, steps_done = 0;
-    float elane = flex_forces_terms<float, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
-    for (int it = 0; it < nsteps && !(st & GRIDFF_REP_NONFINITE); ++it) {
+    Acc elane = flex_forces_terms<Acc, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
+    auto total = [&]() {
+      double ke = 0.0;
+      for (int i = lane; i < n; i += 32) {
+        const double m = __ldg(&tv.body[ab + i]).w;
+        const double vx = s.v[3 * i], vy = s.v[3 * i + 1], vz = s.v[3 * i + 2];
+        ke += 0.5 * m * (vx * vx + vy * vy + vz * vz);
+      }
+      return wsum((double)elane + ke / (double)GRIDFF_ACC);
+    };
+    if (NVE && trace) {
+      const double E = total();
+      if (lane == 0) trace[r] = E;
+    }
+    int rec = 1;
+    for (int it = 0; it < nsteps && (NVE || !(st & GRIDFF_REP_NONFINITE)); ++it) {
       if ((it & 31) == 0) {
         const int sb = stop_bits(ctl, t0, lane);
         if (sb) {
           st |= sb;
           break;
         }
+      }
+      if (NVE) {
+        for (int m = lane; m < 3 * n; m += 32) {
+          const float v = s.v[m] + hdt * GRIDFF_ACC * s_nb[m / 3].w * s.f[m];
+          s.v[m] = v;
+          s.x[m] += dt * v;
+        }
+        elane = flex_forces_terms<Acc, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
+        ++steps_done;
+        for (int m = lane; m < 3 * n; m += 32) s.v[m] += hdt * GRIDFF_ACC * s_nb[m / 3].w * s.f[m];
+        __syncwarp();
+        if (trace && rec_every > 0 && (it + 1) % rec_every == 0) {
+          const double E = total();
+          if (lane == 0) trace[(size_t)rec * trace_stride + r] = E;
+          ++rec;
+        }
+        continue;
       }
       const unsigned long long sstep = (unsigned long long)(step0 + it) * 512ull;
       for (int m = lane; m < 3 * n; m += 32) {
@@ -1834,7 +1648,7 @@ langevin_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tm
         s.x[m] = x + hdt * v;
         s.v[m] = v;
       }
-      elane = flex_forces_terms<float, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
+      elane = flex_forces_terms<Acc, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
       float f2 = 0.f;
       for (int m = lane; m < 3 * n; m += 32) {
         const float rsm = s_nb[m / 3].w;
@@ -1852,94 +1666,13 @@ langevin_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tm
       vs[3 * (size_t)off + m] = s.v[m];
     }
     const double Etot = wsum((double)elane);
-    if (!isfinite(Etot)) st |= GRIDFF_REP_NONFINITE;
+    if (NVE) st |= __reduce_or_sync(kFull, flags);
+    else if (!isfinite(Etot)) st |= GRIDFF_REP_NONFINITE;
     if (lane == 0) {
       status[r] = st;
       energy[r] = Etot;
-      report(ctl, n, steps_done + 1, st, steps_done);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// NVE, flexible replicas: velocity Verlet
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, kMinBlocksPerSM)
-run_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
-                const int* __restrict__ rep_off, int n_rep, float* xs, float* vs, int* status,
-                double* energy, int nsteps, float dt, int rec_every, double* trace, Control ctl,
-                int use_grid, int use_intra, int S) {
-  __shared__ WarpState s_all[kWarpsPerBlock];
-  extern __shared__ __align__(16) unsigned char dyn_smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  WarpState& s = s_all[wib];
-  const StencilCache sc = warp_cache(dyn_smem, S, wib);
-  const int warp = blockIdx.x * kWarpsPerBlock + wib;
-  const int n_warps = gridDim.x * kWarpsPerBlock;
-  const unsigned long long t0 = gtimer();
-  for (int r = warp; r < n_rep; r += n_warps) {
-    const int t = rep_tmpl[r], n = tv.natoms[t], ab = tv.atom_off[t], off = rep_off[r];
-    __syncwarp();
-    cache_reset(sc, lane);
-    for (int k = lane; k < 3 * n; k += 32) {
-      s.x[k] = xs[3 * (size_t)off + k];
-      s.v[k] = vs[3 * (size_t)off + k];
-    }
-    int st = status[r] & ~(GRIDFF_REP_ABORTED | GRIDFF_REP_STEPLIMIT);
-    int flags = 0, evals = 0;
-    double e = flex_forces(g, use_grid, use_intra, tv, ab, n, lane, s, flags, sc);
-    auto total = [&](double epot_lane) {
-      double ke = 0.0;
-      for (int i = lane; i < n; i += 32) {
-        double m = __ldg(&tv.body[ab + i]).w;
-        double vx = s.v[3 * i], vy = s.v[3 * i + 1], vz = s.v[3 * i + 2];
-        ke += 0.5 * m * (vx * vx + vy * vy + vz * vz);
-      }
-      return wsum(epot_lane) + wsum(ke) / (double)GRIDFF_ACC;
-    };
-    double Etot = total(e);
-    if (trace && lane == 0) trace[r] = Etot;
-    int rec = 1;
-    for (int it = 0; it < nsteps; ++it) {
-      if ((it & 31) == 0) {
-        int sb = stop_bits(ctl, t0, lane);
-        if (sb) {
-          st |= sb;
-          break;
-        }
-      }
-      for (int i = lane; i < n; i += 32) {
-        const float h = 0.5f * dt * GRIDFF_ACC / __ldg(&tv.body[ab + i]).w;
-        for (int a = 0; a < 3; ++a) {
-          float vv = s.v[3 * i + a] + h * s.f[3 * i + a];
-          s.v[3 * i + a] = vv;
-          s.x[3 * i + a] += dt * vv;
-        }
-      }
-      e = flex_forces(g, use_grid, use_intra, tv, ab, n, lane, s, flags, sc);
-      ++evals;
-      for (int i = lane; i < n; i += 32) {
-        const float h = 0.5f * dt * GRIDFF_ACC / __ldg(&tv.body[ab + i]).w;
-        for (int a = 0; a < 3; ++a) s.v[3 * i + a] += h * s.f[3 * i + a];
-      }
-      __syncwarp();
-      if (rec_every > 0 && (it + 1) % rec_every == 0) {
-        Etot = total(e);
-        if (trace && lane == 0) trace[(size_t)rec * n_rep + r] = Etot;
-        ++rec;
-      }
-    }
-    __syncwarp();
-    for (int k = lane; k < 3 * n; k += 32) {
-      xs[3 * (size_t)off + k] = s.x[k];
-      vs[3 * (size_t)off + k] = s.v[k];
-    }
-    st |= __reduce_or_sync(kFull, flags);
-    e = wsum(e);
-    if (lane == 0) {
-      status[r] = st;
-      energy[r] = e;
-      report(ctl, n, evals, st & ~GRIDFF_REP_CONVERGED, evals);
+      if (NVE) report(ctl, n, steps_done, st & ~GRIDFF_REP_CONVERGED, steps_done);
+      else report(ctl, n, steps_done + 1, st, steps_done);
     }
   }
 }
@@ -2506,6 +2239,7 @@ LaunchCfg default_launch_cfg(const gridff_replicas* R, bool use_grid) {
     c.queue = 1;
     c.gcache = use_grid ? 1 : 0;
   }
+  c.is_default = true;
   return c;
 }
 
@@ -2526,6 +2260,52 @@ static gridff_status ensure_gcache(gridff_ctx* ctx, gridff_replicas* R) {
     R->gval = nullptr;
     return set_err(ctx, GRIDFF_ENOMEM, "global stencil cache of %d atoms", R->n_atoms);
   }
+  return GRIDFF_OK;
+}
+
+using MdFlexFn = void (*)(GridView, TemplateView, const int*, const int*, const int*, int, float*, float*, int*, double*,
+                          int, float, float, float, float, unsigned long long, long long, int, double*, int, Control, int,
+                          int, int, float4*, int*);
+template <int K, bool GC, bool NVE>
+MdFlexFn md_flex_fn_k(int wpb) {
+  return wpb == 2 ? md_flex_kernel<2, K, GC, NVE> : wpb == 4 ? md_flex_kernel<4, K, GC, NVE> : md_flex_kernel<8, K, GC, NVE>;
+}
+template <bool NVE>
+MdFlexFn md_flex_fn(int wpb, bool f32, bool gc) {
+  if (gc) return f32 ? md_flex_fn_k<REC_F32x4, true, NVE>(wpb) : md_flex_fn_k<-1, true, NVE>(wpb);
+  return f32 ? md_flex_fn_k<REC_F32x4, false, NVE>(wpb) : md_flex_fn_k<-1, false, NVE>(wpb);
+}
+
+// Dynamics of the first n_warp replicas of the cost order, a warp each.
+template <bool NVE>
+gridff_status enqueue_md_flex(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, int n_warp, int nsteps, float dt,
+                              float c1, float c2, float kT_acc, uint64_t seed, int64_t step0, int rec_every, double* trace,
+                              double budget_s, int flags) {
+  cudaStream_t s = ctx->stream;
+  const Control ctl{ctx->ctrl_dev, (unsigned long long)(budget_s > 0 ? budget_s * 1e9 : 0), (DevResult*)ctx->result_dev};
+  const GridView gv = grid ? grid->view() : empty_view();
+  const int use_grid = !(flags & GRIDFF_NO_GRID), use_intra = !(flags & GRIDFF_NO_INTRA);
+  // layout: the replica set's unique-term configuration if it has one
+  const LaunchCfg c = R->cfg.kernel == GRIDFF_KERNEL_FLEX_TERMS ? R->cfg : default_launch_cfg(R, true);
+  const int wpb = c.wpb, S = c.S;
+  bool gc = c.gcache && S == 0 && use_grid;
+  if (gc) {
+    const gridff_status gs = ensure_gcache(ctx, R);
+    if (gs != GRIDFF_OK && !NVE) return gs;
+    gc = gs == GRIDFF_OK;      // NVE runs without the cache where its memory is not to be had
+  }
+  const MdFlexFn fn = md_flex_fn<NVE>(wpb, !grid || grid->kind == REC_F32x4, gc);
+  const size_t dyn = flex_terms_warp_bytes(S) * wpb;
+  GRIDFF_CUDA(ctx, set_dyn_smem((const void*)fn, dyn));
+  int per_sm = 0;
+  GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, 32 * wpb, dyn));
+  if (per_sm < 1) return set_err(ctx, GRIDFF_EINVAL, "dynamics launch does not fit on an SM");
+  const int need = (n_warp + wpb - 1) / wpb;
+  const int blocks = need < per_sm * ctx->n_sm ? need : per_sm * ctx->n_sm;
+  fn<<<blocks, 32 * wpb, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->rep_off, R->order, n_warp, R->x, R->v, R->status, R->energy,
+                                   nsteps, dt, c1, c2, kT_acc, (unsigned long long)seed, (long long)step0, rec_every, trace,
+                                   R->n_rep, ctl, use_grid, use_intra, S, R->gval, R->gkey);
+  GRIDFF_CUDA(ctx, cudaGetLastError());
   return GRIDFF_OK;
 }
 
@@ -2633,6 +2413,8 @@ gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
     win.missProp = cudaAccessPropertyStreaming;
     wp = &win;
   }
+  // flexible batches in the library's own layout: what a team serves faster
+  const FlexSplit sp = c.is_default ? flex_split(ctx, R) : FlexSplit{0, R->n_rep};
   cudaError_t e = cudaSuccess;
   switch (c.kernel) {
     case GRIDFF_KERNEL_RIGID_SUBWARP:
@@ -2656,8 +2438,12 @@ gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
       break;
     case GRIDFF_KERNEL_FLEX_TERMS: {
       const int* ord = c.queue ? (const int*)R->order : nullptr;
-      e = launch_ex(flex_terms_fn(c.wpb, kind, c.gcache != 0), blocks, k.threads, k.dyn, s, wp, gv, R->tv,
-                    (const int*)R->rep_tmpl, (const int*)R->rep_off, ord, R->n_rep, R->x, R->v, R->fire_dt,
+      if (sp.team > 0) {
+        const gridff_status ts = enqueue_team_relax(ctx, grid, R, sp, nsteps, P, flags);
+        if (ts != GRIDFF_OK) return ts;
+      }
+      if (sp.n_warp > 0) e = launch_ex(flex_terms_fn(c.wpb, kind, c.gcache != 0), blocks, k.threads, k.dyn, s, wp, gv, R->tv,
+                    (const int*)R->rep_tmpl, (const int*)R->rep_off, ord, sp.n_warp, R->x, R->v, R->fire_dt,
                     R->fire_alpha, R->fire_nplus, R->status, R->steps, R->energy, R->last_x, R->last_f, nsteps, fp,
                     ctl, use_grid, use_intra, c.S, R->gval, R->gkey);
       break;
@@ -2698,12 +2484,18 @@ gridff_status gridff_eval(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
     dA = Ea_out ? (float*)(p + nE + nF) : nullptr;
     dS = st_out ? (int*)(p + nE + nF + nA) : nullptr;
   }
-  GridView gv = grid ? grid->view() : empty_view();
-  int blocks = persistent_blocks(ctx, (const void*)eval_kernel, R->n_rep);
-  eval_kernel<<<blocks, kThreads, 0, s>>>(gv, R->tv, R->rep_tmpl, R->rep_off, R->n_rep, R->rigid, R->x,
-                                          !(flags & GRIDFF_NO_GRID), !(flags & GRIDFF_NO_INTRA), dE, dF,
-                                          dA, dS);
-  GRIDFF_CUDA(ctx, cudaGetLastError());
+  const int team = eval_team_width(ctx, R);
+  if (team) {
+    const gridff_status ts = enqueue_team_eval(ctx, grid, R, team, dE, dF, dA, dS, flags);
+    if (ts != GRIDFF_OK) return ts;
+  } else {
+    GridView gv = grid ? grid->view() : empty_view();
+    int blocks = persistent_blocks(ctx, (const void*)eval_kernel, R->n_rep);
+    eval_kernel<<<blocks, kThreads, 0, s>>>(gv, R->tv, R->rep_tmpl, R->rep_off, R->order, R->n_rep, R->rigid, R->x,
+                                            !(flags & GRIDFF_NO_GRID), !(flags & GRIDFF_NO_INTRA), dE, dF,
+                                            dA, dS);
+    GRIDFF_CUDA(ctx, cudaGetLastError());
+  }
   if (!dev) {
     GRIDFF_CUDA(ctx, cudaMemcpyAsync(E_out, dE, nE, cudaMemcpyDeviceToHost, s));
     GRIDFF_CUDA(ctx, cudaMemcpyAsync(F_out, dF, nF, cudaMemcpyDeviceToHost, s));
@@ -2813,50 +2605,17 @@ gridff_status gridff_langevin(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
   GRIDFF_CUDA(ctx, cudaSetDevice(ctx->device));
   cudaStream_t s = ctx->stream;
   GRIDFF_CUDA(ctx, cudaMemsetAsync(ctx->result_dev, 0, sizeof(DevResult), s));
-  Control ctl{ctx->ctrl_dev, (unsigned long long)(prm->clock_budget_s > 0 ? prm->clock_budget_s * 1e9 : 0),
-              (DevResult*)ctx->result_dev};
-  GridView gv = grid ? grid->view() : empty_view();
-  const int use_grid = !(flags & GRIDFF_NO_GRID), use_intra = !(flags & GRIDFF_NO_INTRA);
   const double c1 = exp(-(double)prm->gamma * prm->dt);
   const double c2 = sqrt(1.0 - c1 * c1);
   const double kB = 8.617333262e-5;   // eV/K
   const float kT_acc = (float)(kB * prm->temperature * GRIDFF_ACC);
-  // layout: the replica set's unique-term configuration if it has one
-  const LaunchCfg c = R->cfg.kernel == GRIDFF_KERNEL_FLEX_TERMS ? R->cfg : default_launch_cfg(R, true);
-  const int wpb = c.kernel == GRIDFF_KERNEL_FLEX_TERMS ? c.wpb : 8;
-  const int S = c.kernel == GRIDFF_KERNEL_FLEX_TERMS ? c.S : 0;
-  const bool gc = c.kernel == GRIDFF_KERNEL_FLEX_TERMS && c.gcache && S == 0 && use_grid;
-  if (gc) {
-    const gridff_status gs = ensure_gcache(ctx, R);
-    if (gs != GRIDFF_OK) return gs;
-  }
-  using LangevinFn = void (*)(GridView, TemplateView, const int*, const int*, const int*, int, float*, float*, int*,
-                              double*, int, float, float, float, float, unsigned long long, long long, Control, int,
-                              int, int, float4*, int*);
-  const bool f32 = !grid || grid->kind == REC_F32x4;
-  const LangevinFn lf =
-      gc ? (f32 ? (wpb == 2 ? langevin_flex_kernel<2, REC_F32x4, true>
-                            : wpb == 4 ? langevin_flex_kernel<4, REC_F32x4, true> : langevin_flex_kernel<8, REC_F32x4, true>)
-                : (wpb == 2 ? langevin_flex_kernel<2, -1, true>
-                            : wpb == 4 ? langevin_flex_kernel<4, -1, true> : langevin_flex_kernel<8, -1, true>))
-         : (f32 ? (wpb == 2 ? langevin_flex_kernel<2, REC_F32x4, false>
-                            : wpb == 4 ? langevin_flex_kernel<4, REC_F32x4, false>
-                                       : langevin_flex_kernel<8, REC_F32x4, false>)
-                : (wpb == 2 ? langevin_flex_kernel<2, -1, false>
-                            : wpb == 4 ? langevin_flex_kernel<4, -1, false> : langevin_flex_kernel<8, -1, false>));
-  const void* fn = (const void*)lf;
-  const size_t dyn = flex_terms_warp_bytes(S) * wpb;
-  GRIDFF_CUDA(ctx, set_dyn_smem(fn, dyn));
-  int per_sm = 0;
-  GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * wpb, dyn));
-  if (per_sm < 1) return set_err(ctx, GRIDFF_EINVAL, "Langevin launch does not fit on an SM");
-  const int need = (R->n_rep + wpb - 1) / wpb;
-  const int blocks = need < per_sm * ctx->n_sm ? need : per_sm * ctx->n_sm;
   GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev0, s));
-  lf<<<blocks, 32 * wpb, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->rep_off, R->order, R->n_rep, R->x, R->v, R->status,
-                                   R->energy, nsteps, prm->dt, (float)c1, (float)c2, kT_acc,
-                                   (unsigned long long)prm->seed, (long long)prm->step0, ctl, use_grid, use_intra, S,
-                                   R->gval, R->gkey);
+  const FlexSplit sp = flex_split(ctx, R);
+  if (sp.team > 0 && (st = enqueue_team_langevin(ctx, grid, R, sp, nsteps, *prm, (float)c1, (float)c2, kT_acc, flags)) != GRIDFF_OK)
+    return st;
+  if (sp.n_warp > 0 && (st = enqueue_md_flex<false>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, (float)c1, (float)c2, kT_acc,
+                                                    prm->seed, prm->step0, 0, nullptr, prm->clock_budget_s, flags)) != GRIDFF_OK)
+    return st;
   DevResult h{};
   return finish_launch(ctx, &h);
 }
@@ -2888,7 +2647,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
   Control ctl{ctx->ctrl_dev, (unsigned long long)(prm->clock_budget_s > 0 ? prm->clock_budget_s * 1e9 : 0),
               (DevResult*)ctx->result_dev};
   GridView gv = grid ? grid->view() : empty_view();
-  int use_grid = !(flags & GRIDFF_NO_GRID), use_intra = !(flags & GRIDFF_NO_INTRA);
+  const int use_grid = !(flags & GRIDFF_NO_GRID);
   GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev0, s));
   if (R->rigid) {
     if (!use_grid) return set_err(ctx, GRIDFF_EINVAL, "rigid replicas need the grid term");
@@ -2924,13 +2683,11 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
     run_rigid_kernel<<<blocks, kThreads, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->n_rep, R->x, R->v, R->status,
                                                    R->energy, nsteps, prm->dt, rec_every, dtrace, ctl, S);
   } else {
-    const int S = cache_slots(R, false);
-    const size_t dyn = cache_bytes(S) * kWarpsPerBlock;
-    GRIDFF_CUDA(ctx, set_dyn_smem((const void*)run_flex_kernel, dyn));
-    int blocks = persistent_blocks(ctx, (const void*)run_flex_kernel, R->n_rep, dyn);
-    run_flex_kernel<<<blocks, kThreads, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->rep_off, R->n_rep, R->x, R->v,
-                                                  R->status, R->energy, nsteps, prm->dt, rec_every, dtrace, ctl,
-                                                  use_grid, use_intra, S);
+    const FlexSplit sp = flex_split(ctx, R);
+    if (sp.team > 0 && (st = enqueue_team_run(ctx, grid, R, sp, nsteps, *prm, dtrace, flags)) != GRIDFF_OK) return st;
+    if (sp.n_warp > 0 && (st = enqueue_md_flex<true>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, 0.f, 0.f, 0.f, 0, 0, rec_every,
+                                                     dtrace, prm->clock_budget_s, flags)) != GRIDFF_OK)
+      return st;
   }
   DevResult h{};
   gridff_status rs = finish_launch(ctx, &h);

@@ -148,6 +148,9 @@ struct TemplateView {
   const AngleRec* ua;
   const int* ut_off;        // [T+1] unique torsions (TorsionRec, role unused)
   const TorsionRec* ut;
+  const int* gat_off;       // [A+1] slots of the bonded terms whose forces act on an atom
+  const int* gat;           // slot << 1 | negative; a template's slots: bonds (force on i), angles (a, b, c),
+                            // torsions (a, b, c, d), in the order of the unique-term lists
   const int* rot_off;       // [T+1] rotatable bonds
   const Rotor* rot;
   const float4* rigid;      // [T] {M, I1, I2, I3}
@@ -176,6 +179,7 @@ struct LaunchCfg {
   int l2win = 0;     // grid in an L2 persisting access-policy window
   int blocks = 0;    // block cap (0 = every block resident at once)
   int gcache = 0;    // flexible unique-term kernel: stencil cache in global memory
+  bool is_default = false;   // the library's own choice, not a layout given or tuned
 };
 
 struct gridff_replicas {
@@ -187,6 +191,7 @@ struct gridff_replicas {
   int rigid = 0;
   float alpha = 1.5f;
   int max_natoms = 0;
+  int max_slots = 0;        // bonded-term slots of the largest template (flexible)
   // device
   void* tmpl_blob = nullptr;   // one allocation holding every template array
   TemplateView tv{};
@@ -233,6 +238,23 @@ gridff_status enqueue_build_poses(gridff_replicas* R, const float* d_poses, int 
 gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, const LaunchCfg& c,
                             int blocks, int nsteps, const gridff_fire_params& P, int flags);
 gridff_status check_fire_params(gridff_ctx* ctx, const gridff_fire_params& P);
+// Flexible batches: the first n_warp replicas of the cost order by the
+// warp-per-replica kernels, the others by teams of `team` warps (flex_team.cu).
+struct FlexSplit {
+  int team;
+  int n_warp;
+};
+FlexSplit flex_split(const gridff_ctx* ctx, const gridff_replicas* R);
+int eval_team_width(const gridff_ctx* ctx, const gridff_replicas* R);   // 0: a warp per replica
+// Enqueued on the context stream.
+gridff_status enqueue_team_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, FlexSplit sp, int nsteps,
+                                 const gridff_fire_params& P, int flags);
+gridff_status enqueue_team_langevin(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, FlexSplit sp, int nsteps,
+                                    const gridff_langevin_params& P, float c1, float c2, float kT_acc, int flags);
+gridff_status enqueue_team_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, FlexSplit sp, int nsteps,
+                               const gridff_md_params& P, double* trace, int flags);
+gridff_status enqueue_team_eval(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, int NW, double* E, float* F,
+                                float* Ea, int* st, int flags);
 // Binned point evaluation (points.cu): device arrays, enqueued on the
 // context stream (gridff_eval_points with GRIDFF_POINTS_BINNED).
 gridff_status enqueue_eval_points_binned(gridff_ctx* ctx, const gridff_grid* grid, int64_t n, const float* xyz,

@@ -204,6 +204,7 @@ gridff_status gridff_tune(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
   };
 
   LaunchCfg best = default_launch_cfg(R, use_grid);
+  best.is_default = false;   // trials are layouts of gridff_launch_config
   double best_rate = 0;
   st = trial(best, best_rate);
   for (int pass = 0; pass < 2 && st == GRIDFF_OK; ++pass) {

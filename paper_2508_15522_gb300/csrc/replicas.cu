@@ -210,6 +210,8 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
   std::vector<BondTerm> ub;
   std::vector<AngleRec> ua;
   std::vector<TorsionRec> ut;
+  std::vector<int> gat_off(1, 0), gat;
+  int max_slots = 0;
   std::vector<double> tmpl_cost(n_templates);
   std::vector<int> rot_off(1, 0);
   std::vector<Rotor> rot;
@@ -280,6 +282,22 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
     tub = spread_terms(tub, 2, [](const BondTerm& b, int r) { return r == 0 ? b.i : b.j; });
     tua = spread_terms(tua, 3, [](const AngleRec& a, int r) { return r == 0 ? a.a : r == 1 ? a.b : a.c; });
     tut = spread_terms(tut, 4, [](const TorsionRec& q, int r) { return r == 0 ? q.a : r == 1 ? q.b : r == 2 ? q.c : q.d; });
+    // slots of the terms' forces, and per atom those that act on it
+    std::vector<std::vector<int>> acts(n);
+    int slot = 0;
+    for (auto& b : tub) {
+      acts[b.i].push_back(slot << 1);
+      acts[b.j].push_back(slot++ << 1 | 1);
+    }
+    for (auto& a : tua)
+      for (int i : {a.a, a.b, a.c}) acts[i].push_back(slot++ << 1);
+    for (auto& q : tut)
+      for (int i : {q.a, q.b, q.c, q.d}) acts[i].push_back(slot++ << 1);
+    max_slots = std::max(max_slots, slot);
+    for (auto& a : acts) {
+      gat.insert(gat.end(), a.begin(), a.end());
+      gat_off.push_back((int)gat.size());
+    }
     ub.insert(ub.end(), tub.begin(), tub.end());
     ua.insert(ua.end(), tua.begin(), tua.end());
     ut.insert(ut.end(), tut.begin(), tut.end());
@@ -376,7 +394,7 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
          o_a = push(blob, angles), o_tof = push(blob, tors_off), o_t = push(blob, tors),
          o_rig = push(blob, rig), o_rmax = push(blob, rmax), o_ubo = push(blob, ub_off), o_ub = push(blob, ub), o_uao = push(blob, ua_off),
          o_ua = push(blob, ua), o_uto = push(blob, ut_off), o_ut = push(blob, ut), o_ord = push(blob, order),
-         o_roff = push(blob, rot_off), o_rot = push(blob, rot);
+         o_roff = push(blob, rot_off), o_rot = push(blob, rot), o_goff = push(blob, gat_off), o_gat = push(blob, gat);
   gridff_replicas* R = new gridff_replicas();
   R->ctx = ctx;
   R->device = ctx->device;
@@ -386,6 +404,7 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
   R->rigid = rigid ? 1 : 0;
   R->alpha = (float)alpha;
   R->max_natoms = max_n;
+  R->max_slots = max_slots;
   auto bail = [&](gridff_status st, const char* what) {
     gridff_replicas_destroy(R);
     return set_err(ctx, st, "%s", what);
@@ -415,6 +434,8 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
   R->tv.ut_off = (const int*)(B + o_uto);
   R->tv.ut = (const TorsionRec*)(B + o_ut);
   R->order = (int*)(B + o_ord);
+  R->tv.gat_off = (const int*)(B + o_goff);
+  R->tv.gat = (const int*)(B + o_gat);
   R->tv.rot_off = (const int*)(B + o_roff);
   R->tv.rot = (const Rotor*)(B + o_rot);
   R->h_rot_off = new int[n_templates + 1];
