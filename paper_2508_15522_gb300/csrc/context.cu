@@ -48,6 +48,15 @@ gridff_status gridff_create(int device, void* cuda_stream, gridff_ctx** out) {
   if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) return fail(GRIDFF_ECUDA);
   ctx->ctrl_dev = (int*)d;
   if (cudaMalloc(&ctx->result_dev, 64) != cudaSuccess) return fail(GRIDFF_ENOMEM);
+  if (cudaHostAlloc(&ctx->result_host, 64, cudaHostAllocDefault) != cudaSuccess) return fail(GRIDFF_ENOMEM);
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  uint64_t kept = kScratchKept;
+  if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &kept) != cudaSuccess)
+    return fail(GRIDFF_ENOMEM);
   if (cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess)
     return fail(GRIDFF_ECUDA);
   *out = ctx;
@@ -67,6 +76,8 @@ void gridff_destroy(gridff_ctx* ctx) {
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
   if (ctx->ev1) cudaEventDestroy(ctx->ev1);
   if (ctx->result_dev) cudaFree(ctx->result_dev);
+  if (ctx->result_host) cudaFreeHost(ctx->result_host);
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   if (ctx->ctrl_host) cudaFreeHost((void*)ctx->ctrl_host);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   cudaGetLastError();   // leave no error of this teardown behind

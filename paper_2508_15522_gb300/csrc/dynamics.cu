@@ -2198,9 +2198,10 @@ KernelShape shape_of(const gridff_replicas* R, const LaunchCfg& c, int kind) {
 gridff_status finish_launch(gridff_ctx* ctx, DevResult* hres) {
   GRIDFF_CUDA(ctx, cudaGetLastError());
   GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
-  GRIDFF_CUDA(ctx, cudaMemcpyAsync(hres, ctx->result_dev, sizeof(DevResult), cudaMemcpyDeviceToHost,
+  GRIDFF_CUDA(ctx, cudaMemcpyAsync(ctx->result_host, ctx->result_dev, sizeof(DevResult), cudaMemcpyDeviceToHost,
                                    ctx->stream));
   GRIDFF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  *hres = *(const DevResult*)ctx->result_host;
   float ms = 0.f;
   GRIDFF_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
   ctx->last_ms = ms;
@@ -2477,7 +2478,7 @@ gridff_status gridff_eval(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
   float* dA = Ea_out;
   int* dS = st_out;
   if (!dev) {
-    GRIDFF_CUDA(ctx, cudaMallocAsync(&stg.ptr, nE + nF + nA + nS + 64, s));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &stg.ptr, nE + nF + nA + nS + 64));
     char* p = (char*)stg.ptr;
     dE = (double*)p;
     dF = (float*)(p + nE);
@@ -2522,7 +2523,7 @@ gridff_status gridff_eval_points(gridff_ctx* ctx, const gridff_grid* grid, int64
   float *dE = E, *dF = F;
   int* dS = status;
   if (!dev) {
-    GRIDFF_CUDA(ctx, cudaMallocAsync(&stg.ptr, 3 * n3 + 2 * n1 + 64, s));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &stg.ptr, 3 * n3 + 2 * n1 + 64));
     char* p = (char*)stg.ptr;
     float* hx = (float*)p;
     float* hq = (float*)(p + n3);
@@ -2639,7 +2640,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
     if (dev) {
       dtrace = energy_trace;
     } else {
-      GRIDFF_CUDA(ctx, cudaMallocAsync(&stg.ptr, tbytes, s));
+      GRIDFF_CUDA(ctx, scratch_alloc(ctx, &stg.ptr, tbytes));
       dtrace = (double*)stg.ptr;
     }
   }

@@ -575,7 +575,7 @@ gridff_status pack_records(gridff_ctx* ctx, gridff_grid* g, const double* data) 
   g->scale[0] = g->scale[1] = g->scale[2] = 1.f;
   if (g->storage != GRIDFF_STORE_F32) {
     unsigned long long* mx = nullptr;
-    GRIDFF_CUDA(ctx, cudaMallocAsync((void**)&mx, 3 * sizeof(unsigned long long), s));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &mx, 3 * sizeof(unsigned long long)));
     cudaError_t e = cudaMemsetAsync(mx, 0, 3 * sizeof(unsigned long long), s);
     if (e == cudaSuccess) {
       absmax_kernel<<<4 * ctx->n_sm, 256, 0, s>>>(data, (size_t)nx * ny * nz, nch, mx);

@@ -61,6 +61,8 @@ struct gridff_ctx {
   int l2_limit_set = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   double last_ms = 0.0;
+  cudaMemPool_t pool = nullptr;       // scratch of the calls (scratch_alloc)
+  void* result_host = nullptr;        // pinned copy of result_dev
   std::string err;
 };
 
@@ -218,6 +220,17 @@ struct gridff_replicas {
   Rotor* h_rot = nullptr;
   LaunchCfg cfg;               // set by gridff_tune / gridff_set_launch_config
 };
+
+// Stream-ordered scratch of a call, freed with cudaFreeAsync on the context
+// stream.  From the context's own pool, which keeps up to kScratchKept bytes
+// between calls (the default pool returns everything at every
+// synchronisation, so each call mapped its scratch anew: 0.3 ms) and is
+// destroyed with the context.
+constexpr size_t kScratchKept = (size_t)256 << 20;
+template <class T>
+cudaError_t scratch_alloc(gridff_ctx* ctx, T** p, size_t bytes) {
+  return cudaMallocFromPoolAsync((void**)p, bytes, ctx->pool, ctx->stream);
+}
 
 // error helpers -------------------------------------------------------------
 gridff_status set_err(gridff_ctx* ctx, gridff_status st, const char* fmt, ...);

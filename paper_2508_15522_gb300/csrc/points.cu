@@ -298,7 +298,7 @@ gridff_status enqueue_eval_points_binned(gridff_ctx* ctx, const gridff_grid* gri
   const size_t b_counts = ((size_t)nb * 4 + 255) & ~size_t(255), b_tiles = ((size_t)n_tiles * 4 + 255) & ~size_t(255),
                b_kr = ((size_t)ni * 8 + 255) & ~size_t(255), b_sorted = (size_t)ni * sizeof(SortedPoint);
   char* scratch = nullptr;
-  GRIDFF_CUDA(ctx, cudaMallocAsync((void**)&scratch, 2 * b_counts + b_tiles + b_kr + b_sorted, s));
+  GRIDFF_CUDA(ctx, scratch_alloc(ctx, &scratch, 2 * b_counts + b_tiles + b_kr + b_sorted));
   int* counts = (int*)scratch;
   int* start = (int*)(scratch + b_counts);
   int* tiles = (int*)(scratch + 2 * b_counts);

@@ -373,7 +373,7 @@ gridff_status gridff_build_poses(gridff_replicas* R, const float* poses, const d
   const float* d = poses;
   void* tmp = nullptr;
   if (!(flags & GRIDFF_DEVICE_PTRS)) {
-    GRIDFF_CUDA(ctx, cudaMallocAsync(&tmp, bytes, s));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &tmp, bytes));
     const cudaError_t e = cudaMemcpyAsync(tmp, poses, bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(tmp, s);
@@ -422,7 +422,7 @@ gridff_status gridff_pose_targets(const gridff_replicas* R, const double origin_
   float *dt = targets, *dm = tors_mask;
   void* tmp = nullptr;
   if (!dev) {
-    GRIDFF_CUDA(ctx, cudaMallocAsync(&tmp, tb + mb, s));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &tmp, tb + mb));
     dt = (float*)tmp;
     dm = tors_mask ? (float*)((char*)tmp + tb) : nullptr;
   }

@@ -563,7 +563,7 @@ gridff_status gridff_get_positions(gridff_replicas* R, float* x, int flags) {
   float* dst = x;
   float* tmp = nullptr;
   if (!(flags & GRIDFF_DEVICE_PTRS)) {
-    GRIDFF_CUDA(ctx, cudaMallocAsync(&tmp, bytes, ctx->stream));
+    GRIDFF_CUDA(ctx, scratch_alloc(ctx, &tmp, bytes));
     dst = tmp;
   }
   rigid_positions_kernel<<<R->n_rep, 64, 0, ctx->stream>>>(R->tv, R->rep_tmpl, R->rep_off, R->x,

@@ -214,7 +214,7 @@ gridff_status gridff_rmsd_unique(gridff_replicas* R, int32_t tmpl, int32_t n, co
   const size_t pose_bytes = 7 * (size_t)n * sizeof(float), dup_bytes = (size_t)n * sizeof(int32_t);
   char* buf = nullptr;
   const size_t mom_off = 0, pose_off = 256, dup_off = pose_off + ((pose_bytes + 255) & ~(size_t)255);
-  GRIDFF_CUDA(ctx, cudaMallocAsync((void**)&buf, dup_off + dup_bytes, s));
+  GRIDFF_CUDA(ctx, scratch_alloc(ctx, &buf, dup_off + dup_bytes));
   Moments* mom = (Moments*)(buf + mom_off);
   const float* p = dev ? poses : (const float*)(buf + pose_off);
   int* d = dev ? dup_of : (int*)(buf + dup_off);
@@ -253,7 +253,7 @@ extern "C" gridff_status gridff_rmsd_unique_xyz(gridff_ctx* ctx, int32_t na, int
   const size_t cen_off = 0, xyz_off = ((size_t)n * sizeof(float2) + 255) & ~(size_t)255;
   const size_t dup_off = xyz_off + ((xyz_bytes + 255) & ~(size_t)255);
   char* buf = nullptr;
-  GRIDFF_CUDA(ctx, cudaMallocAsync((void**)&buf, dup_off + dup_bytes, s));
+  GRIDFF_CUDA(ctx, scratch_alloc(ctx, &buf, dup_off + dup_bytes));
   const float* p = dev ? xyz : (const float*)(buf + xyz_off);
   int* d = dev ? dup_of : (int*)(buf + dup_off);
   float2* cen = (float2*)(buf + cen_off);
