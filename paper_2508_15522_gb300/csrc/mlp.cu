@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "mlp_fused.cuh"
 #include "trace.h"
 
 namespace {
@@ -468,6 +469,13 @@ struct gridff_mlp {
   int loss_cap = 0;
   long long rng_step = 0;
   StepCounters* ctr = nullptr;     // device step counters of the training loop
+  // four-launch form (mlp_fused.cuh): operands in fragment order and workspaces
+  bool fused = false;
+  std::vector<__nv_bfloat16*> Wf, Wr;
+  char* fbuf = nullptr;            // inputs and outputs of fcap rows
+  int fcap = 0;
+  char* tbuf = nullptr;            // training workspace of tcap padded rows
+  int tcap = 0;
 };
 
 namespace {
@@ -548,12 +556,164 @@ void gemm(cudaStream_t s, const __nv_bfloat16* A, int lda, const __nv_bfloat16* 
   splitk_sum_kernel<<<grid1((long long)M * N), 256, 0, s>>>(part, cstride, S, M, N, ldc, C);
 }
 
-void refresh_bf16(gridff_mlp* m) {
+// The four-launch form covers the network (a training batch also needs
+// K <= 240 proposals per target: a block evaluates them together).
+bool fused_shape(const gridff_mlp* m) {
+  return m->L <= kFusedMaxL && *std::max_element(m->pads.begin(), m->pads.end()) <= kFusedW;
+}
+bool fused_train(const gridff_mlp* m, int K) { return m->fused && 2 * K + 15 <= kLossMax; }
+
+FusedNet fused_net(gridff_mlp* m, int rows) {
+  FusedNet f{};
+  f.L = m->L;
+  f.rows = rows;
+  f.Mp = pad16(rows);
+  for (int l = 0; l <= m->L; ++l) {
+    f.size[l] = m->sizes[l];
+    f.pad[l] = m->pads[l];
+  }
+  for (int l = 0; l < m->L; ++l) {
+    f.woff[l] = m->woff[l];
+    f.boff[l] = m->boff[l];
+    f.Wf[l] = m->Wf[l];
+    f.Wr[l] = m->Wr[l];
+  }
+  f.P = m->P;
+  f.Gr = m->Gr;
+  f.Am = m->Am;
+  f.Av = m->Av;
+  return f;
+}
+
+size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+gridff_status grow(gridff_mlp* m, char** buf, int* cap, int rows, size_t bytes) {
+  if (rows <= *cap) return GRIDFF_OK;
+  gridff_ctx* ctx = m->ctx;
+  if (*buf) {
+    GRIDFF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    cudaFree(*buf);
+    m->owned.erase(std::remove(m->owned.begin(), m->owned.end(), (void*)*buf), m->owned.end());
+    *buf = nullptr;
+    *cap = 0;
+  }
+  if (dalloc(m, buf, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return set_err(ctx, GRIDFF_ENOMEM, "MLP workspace for %d rows", rows);
+  }
+  *cap = rows;
+  return GRIDFF_OK;
+}
+
+// Inputs Xs [rows][n_in] and outputs Y [rows][n_out].
+gridff_status fused_io(gridff_mlp* m, int rows, FusedNet& f, float** Xs) {
+  const size_t bx = up256((size_t)rows * m->sizes[0] * sizeof(float)), by = up256((size_t)rows * kOut * sizeof(float));
+  const gridff_status st = grow(m, &m->fbuf, &m->fcap, rows, bx + by);
+  if (st != GRIDFF_OK) return st;
+  const size_t cx = up256((size_t)m->fcap * m->sizes[0] * sizeof(float));
+  *Xs = (float*)m->fbuf;
+  f.Y = (float*)(m->fbuf + cx);
+  return GRIDFF_OK;
+}
+
+// Workspace of a training step; targets and masks staged from the host at Ts, Ms.
+gridff_status fused_workspace(gridff_mlp* m, int rows, FusedNet& f, FusedLoss& q, float** Ts, float** Ms) {
+  for (int pass = 0; pass < 2; ++pass) {
+    const size_t Mp = pass ? (size_t)m->tcap : (size_t)f.Mp;
+    size_t o = 0;
+    char* b = m->tbuf;
+    auto take = [&](size_t bytes) {
+      char* p = b ? b + o : nullptr;
+      o += up256(bytes);
+      return p;
+    };
+    *Ts = (float*)take(Mp * kOut * 4);
+    *Ms = (float*)take(Mp * kTors * 4);
+    q.loss = (float*)take(Mp * 4);
+    q.winner = (int*)take(Mp * 4);
+    for (int l = 0; l < m->L; ++l) {
+      const size_t ip = m->pads[l], op = m->pads[l + 1];
+      f.H[l] = (__nv_bfloat16*)take(Mp * ip * 2);
+      f.Gf[l] = (float*)take(Mp * op * 4);
+      f.Gb[l] = (__nv_bfloat16*)take(Mp * op * 2);
+      f.part[l] = (float*)take(kMaxSplit * op * ip * 4);
+      f.dbp[l] = (float*)take(64 * op * 4);
+    }
+    if (!pass) {
+      const gridff_status st = grow(m, &m->tbuf, &m->tcap, f.Mp, o);
+      if (st != GRIDFF_OK) return st;
+    }
+  }
+  // split of the weight gradients' rows (as the layer-by-layer products take it)
+  for (int l = 0; l < m->L; ++l) {
+    f.S[l] = 1;
+    if ((long long)(m->pads[l + 1] / 16) * (m->pads[l] / 8) < 2048)
+      for (int cand = kMaxSplit; cand > 1; cand >>= 1)
+        if ((f.Mp / 16) % cand == 0 && f.Mp / cand >= 128) {
+          f.S[l] = cand;
+          break;
+        }
+  }
+  f.rpc = std::max(256, (f.Mp + 63) / 64);
+  f.chunks = (f.Mp + f.rpc - 1) / f.rpc;
+  return GRIDFF_OK;
+}
+
+void fused_forward(gridff_mlp* m, const FusedNet& f, const FusedInput& in, int train) {
+  // 64 rows a block re-read the weights a quarter as often and need enough
+  // rows for the chip
+  const bool wide = f.rows >= 8192;
+  const int per = wide ? 64 : 16;
+  const size_t dyn = 2 * (size_t)per * kFusedLd * sizeof(__nv_bfloat16);
+  auto fn = wide ? fused_forward_kernel<4> : fused_forward_kernel<1>;
+  if (wide) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  fn<<<(f.Mp + per - 1) / per, 256, dyn, m->ctx->stream>>>(f, in, train);
+}
+
+// One training step: forward, loss and backward, gradients, update; hist: slot
+// of the step's mean loss, or null.  Enqueued, no synchronisation.
+gridff_status fused_step(gridff_mlp* m, const FusedNet& f, const FusedInput& in, const FusedLoss& q,
+                         const gridff_train_params* tp, long long t, int update, float* hist) {
+  cudaStream_t s = m->ctx->stream;
+  fused_forward(m, f, in, 1);
+  fused_backward_kernel<<<f.Mp / 16, 256, 0, s>>>(f, q);
+  GradMap g{};
+  int n = 0;
+  for (int l = 0; l < f.L; ++l) {
+    g.first[l] = n;
+    g.tx[l] = (f.pad[l] + 63) / 64;
+    g.ty[l] = (f.pad[l + 1] + 63) / 64;
+    n += g.tx[l] * g.ty[l] * f.S[l];
+  }
+  g.first[f.L] = n;
+  for (int l = 0; l < f.L; ++l) {
+    g.db_first[l] = n - g.first[f.L];
+    n += (f.size[l + 1] + 31) / 32 * f.chunks;
+  }
+  g.db_first[f.L] = n - g.first[f.L];
+  fused_grad_kernel<<<n, 128, 0, s>>>(f, g);
+  AdamArgs ad{tp->beta1, tp->beta2, tp->eps, 0.f, 0.f, update};
+  if (update) {
+    ad.c1 = (float)(tp->lr / (1.0 - pow((double)tp->beta1, (double)t)));
+    ad.c2 = (float)(1.0 / (1.0 - pow((double)tp->beta2, (double)t)));
+  }
+  fused_update_kernel<<<grid1((long long)m->n_params) + 1, 256, 0, s>>>(f, ad, (int)m->n_params, q.loss, q.n_targets, hist);
+  GRIDFF_CUDA(m->ctx, cudaGetLastError());
+  return GRIDFF_OK;
+}
+
+void refresh_layers(gridff_mlp* m) {
   for (int l = 0; l < m->L; ++l) {
     const int in = m->sizes[l], out = m->sizes[l + 1], ip = m->pads[l], op = m->pads[l + 1];
     weights_bf16_kernel<<<grid1((long long)op * ip), 256, 0, m->ctx->stream>>>(m->P + m->woff[l], out, in, op,
                                                                                 ip, m->Wb[l], m->WbT[l]);
   }
+}
+
+// The operands of the form that runs, from the FP32 parameters.
+void refresh_bf16(gridff_mlp* m) {
+  if (!m->fused) return refresh_layers(m);
+  fused_weights_kernel<<<grid1((long long)m->n_params), 256, 0, m->ctx->stream>>>(fused_net(m, 16), (int)m->n_params);
 }
 
 // Forward of `rows` rows whose layer-0 input is already in H[0]/HT[0].
@@ -579,6 +739,7 @@ gridff_status enqueue_train(gridff_mlp* m, int n_targets, int K, bool mask_on, c
   cudaStream_t s = ctx->stream;
   const int rows = n_targets * K;
   const int Mp = pad16(rows), L = m->L;
+  if (m->fused && !ctr) refresh_layers(m);   // (a captured loop's caller did it before the capture)
   forward_rows(m, rows);
   // loss and dL/dY (written into G with the last layer's padded stride)
   const int op_last = m->pads[L];
@@ -626,7 +787,8 @@ gridff_status enqueue_train(gridff_mlp* m, int n_targets, int K, bool mask_on, c
                                                                         reinterpret_cast<const char*>(ctr) +
                                                                         offsetof(StepCounters, c12))
                                                                   : nullptr);
-    refresh_bf16(m);
+    refresh_layers(m);
+    if (m->fused) refresh_bf16(m);
   }
   return GRIDFF_OK;
 }
@@ -661,8 +823,19 @@ gridff_status gridff_mlp_create(gridff_ctx* ctx, int32_t n_layers, const int32_t
   bool ok = dalloc(m, &m->P, off) == cudaSuccess && dalloc(m, &m->Gr, off) == cudaSuccess &&
             dalloc(m, &m->Am, off) == cudaSuccess && dalloc(m, &m->Av, off) == cudaSuccess &&
             dalloc(m, &m->desc, (size_t)sizes[0]) == cudaSuccess;
+  m->fused = fused_shape(m);
   m->Wb.assign(n_layers, nullptr);
   m->WbT.assign(n_layers, nullptr);
+  m->Wf.assign(n_layers, nullptr);
+  m->Wr.assign(n_layers, nullptr);
+  for (int l = 0; l < n_layers && ok && m->fused; ++l) {
+    const size_t nf = (size_t)m->pads[l + 1] * 32 * k32(m->pads[l]), nr = (size_t)m->pads[l] * 32 * k32(m->pads[l + 1]);
+    ok &= dalloc(m, &m->Wf[l], nf) == cudaSuccess && dalloc(m, &m->Wr[l], nr) == cudaSuccess;
+    if (ok) {
+      cudaMemsetAsync(m->Wf[l], 0, nf * sizeof(__nv_bfloat16), ctx->stream);
+      cudaMemsetAsync(m->Wr[l], 0, nr * sizeof(__nv_bfloat16), ctx->stream);
+    }
+  }
   for (int l = 0; l < n_layers && ok; ++l) {
     ok &= dalloc(m, &m->Wb[l], (size_t)m->pads[l] * m->pads[l + 1]) == cudaSuccess;
     ok &= dalloc(m, &m->WbT[l], (size_t)m->pads[l] * m->pads[l + 1]) == cudaSuccess;
@@ -726,6 +899,18 @@ gridff_status gridff_mlp_forward(gridff_mlp* m, int32_t rows, const float* x, fl
   if (!m || !x || !y || rows < 1) return set_err(m ? m->ctx : nullptr, GRIDFF_EINVAL, "bad argument");
   gridff_ctx* ctx = m->ctx;
   GRIDFF_CUDA(ctx, cudaSetDevice(ctx->device));
+  if (m->fused) {
+    FusedNet f = fused_net(m, rows);
+    float* Xs = nullptr;
+    const gridff_status fs = fused_io(m, rows, f, &Xs);
+    if (fs != GRIDFF_OK) return fs;
+    GRIDFF_CUDA(ctx, cudaMemcpyAsync(Xs, x, (size_t)rows * m->sizes[0] * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
+    fused_forward(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, 0);
+    GRIDFF_CUDA(ctx, cudaGetLastError());
+    GRIDFF_CUDA(ctx, cudaMemcpyAsync(y, f.Y, (size_t)rows * kOut * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
+    GRIDFF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return GRIDFF_OK;
+  }
   gridff_status st = ensure_batch(m, rows);
   if (st != GRIDFF_OK) return st;
   cudaStream_t s = ctx->stream;
@@ -749,20 +934,44 @@ gridff_status gridff_mlp_train_step(gridff_mlp* m, int32_t n_targets, int32_t K,
   gridff_ctx* ctx = m->ctx;
   GRIDFF_CUDA(ctx, cudaSetDevice(ctx->device));
   const int rows = n_targets * K;
-  gridff_status st = ensure_batch(m, std::max(rows, n_targets));
-  if (st != GRIDFF_OK) return st;
   cudaStream_t s = ctx->stream;
   const int Mp = pad16(rows), n_in = m->sizes[0];
-  GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->Xs, x, (size_t)rows * n_in * sizeof(float), cudaMemcpyHostToDevice, s));
-  GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->Ts, targets, (size_t)n_targets * kOut * sizeof(float), cudaMemcpyHostToDevice, s));
+  const bool fused = fused_train(m, K);
+  FusedNet f = fused_net(m, rows);
+  FusedLoss q{};
+  float *Xs = m->Xs, *Ts = m->Ts, *Ms = m->Ms;
+  gridff_status st = fused ? fused_io(m, rows, f, &Xs) : ensure_batch(m, std::max(rows, n_targets));
+  if (st == GRIDFF_OK && fused) st = fused_workspace(m, rows, f, q, &Ts, &Ms);
+  if (st != GRIDFF_OK) return st;
+  if (!fused) {
+    Xs = m->Xs;
+    Ts = m->Ts;
+    Ms = m->Ms;
+    q.loss = m->loss;
+  }
+  GRIDFF_CUDA(ctx, cudaMemcpyAsync(Xs, x, (size_t)rows * n_in * sizeof(float), cudaMemcpyHostToDevice, s));
+  GRIDFF_CUDA(ctx, cudaMemcpyAsync(Ts, targets, (size_t)n_targets * kOut * sizeof(float), cudaMemcpyHostToDevice, s));
   if (tors_mask)
-    GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->Ms, tors_mask, (size_t)n_targets * kTors * sizeof(float),
-                                     cudaMemcpyHostToDevice, s));
-  input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->Xs, rows, n_in, Mp, m->pads[0], m->H[0], m->HT[0]);
-  if ((st = enqueue_train(m, n_targets, K, tors_mask != nullptr, tp, flags)) != GRIDFF_OK) return st;
+    GRIDFF_CUDA(ctx, cudaMemcpyAsync(Ms, tors_mask, (size_t)n_targets * kTors * sizeof(float), cudaMemcpyHostToDevice, s));
+  if (fused) {
+    q.T = Ts;
+    q.mask = tors_mask ? Ms : nullptr;
+    q.n_targets = n_targets;
+    q.K = K;
+    q.w_q = tp->w_q;
+    q.w_t = tp->w_t;
+    q.tile_x = (float)tp->tile[0];
+    q.tile_y = (float)tp->tile[1];
+    const int update = !(flags & GRIDFF_MLP_NO_UPDATE);
+    m->t += update;
+    if ((st = fused_step(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, q, tp, m->t, update, nullptr)) != GRIDFF_OK) return st;
+  } else {
+    input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->Xs, rows, n_in, Mp, m->pads[0], m->H[0], m->HT[0]);
+    if ((st = enqueue_train(m, n_targets, K, tors_mask != nullptr, tp, flags)) != GRIDFF_OK) return st;
+  }
   if (loss_out) {
     std::vector<float> l(n_targets);
-    GRIDFF_CUDA(ctx, cudaMemcpyAsync(l.data(), m->loss, n_targets * sizeof(float), cudaMemcpyDeviceToHost, s));
+    GRIDFF_CUDA(ctx, cudaMemcpyAsync(l.data(), q.loss, n_targets * sizeof(float), cudaMemcpyDeviceToHost, s));
     GRIDFF_CUDA(ctx, cudaStreamSynchronize(s));
     double sum = 0;
     for (float v : l) sum += v;
@@ -811,7 +1020,12 @@ gridff_status gridff_mlp_train(gridff_mlp* m, int32_t steps, int32_t n_targets, 
   if ((long long)n_targets * K >= (1 << 20)) return set_err(ctx, GRIDFF_EINVAL, "batch rows must be below 2^20");
   GRIDFF_CUDA(ctx, cudaSetDevice(ctx->device));
   const int rows = n_targets * K;
-  gridff_status st = ensure_batch(m, rows);
+  const bool fused = fused_train(m, K);
+  FusedNet f = fused_net(m, rows);
+  FusedLoss q{};
+  float *Xs = nullptr, *Ts = nullptr, *Ms = nullptr;
+  gridff_status st = fused ? fused_io(m, rows, f, &Xs) : ensure_batch(m, rows);
+  if (st == GRIDFF_OK && fused) st = fused_workspace(m, rows, f, q, &Ts, &Ms);
   if (st != GRIDFF_OK) return st;
   if (steps > m->loss_cap) {
     if (m->loss_hist) {
@@ -823,11 +1037,35 @@ gridff_status gridff_mlp_train(gridff_mlp* m, int32_t steps, int32_t n_targets, 
     if (dalloc(m, &m->loss_hist, (size_t)steps) != cudaSuccess) return set_err(ctx, GRIDFF_ENOMEM, "loss history");
     m->loss_cap = steps;
   }
-  if (!m->ctr && dalloc(m, &m->ctr, 1) != cudaSuccess) return set_err(ctx, GRIDFF_ENOMEM, "step counters");
   cudaStream_t s = ctx->stream;
   const int Mp = pad16(rows);
   if (n_desc > 0)
     GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->desc, descriptor, n_desc * sizeof(float), cudaMemcpyHostToDevice, s));
+  if (fused) {
+    q.T = m->T_all;
+    q.mask = m->M_all;
+    q.n_all = m->n_all;
+    q.n_targets = n_targets;
+    q.K = K;
+    q.seed = (unsigned long long)seed;
+    q.w_q = tp->w_q;
+    q.w_t = tp->w_t;
+    q.tile_x = (float)tp->tile[0];
+    q.tile_y = (float)tp->tile[1];
+    for (int k = 0; k < steps; ++k) {
+      q.base = (unsigned long long)(m->rng_step + k) << 20;
+      const FusedInput in{nullptr, m->desc, n_desc, (unsigned long long)seed, q.base};
+      if ((st = fused_step(m, f, in, q, tp, m->t + k + 1, 1, m->loss_hist + k)) != GRIDFF_OK) return st;
+    }
+    m->rng_step += steps;
+    m->t += steps;
+    if (losses && steps > 0)
+      GRIDFF_CUDA(ctx, cudaMemcpyAsync(losses, m->loss_hist, steps * sizeof(float), cudaMemcpyDeviceToHost, s));
+    GRIDFF_CUDA(ctx, cudaStreamSynchronize(s));
+    return GRIDFF_OK;
+  }
+  if (!m->ctr && dalloc(m, &m->ctr, 1) != cudaSuccess) return set_err(ctx, GRIDFF_ENOMEM, "step counters");
+  if (m->fused) refresh_layers(m);
   // The loop is launch-bound (about 45 small launches per step), so one step
   // is captured in a CUDA graph and replayed `steps` times; everything that
   // changes between steps (random-stream step, history slot, Adam t and its
@@ -881,20 +1119,26 @@ gridff_status gridff_mlp_propose(gridff_mlp* m, gridff_replicas* R, const float*
   if (!(tile_xy[0] > 0 && tile_xy[1] > 0)) return set_err(ctx, GRIDFF_EINVAL, "tile lengths must be positive");
   GRIDFF_CUDA(ctx, cudaSetDevice(ctx->device));
   const int rows = R->n_rep;
-  gridff_status st = ensure_batch(m, rows);
+  FusedNet f = fused_net(m, rows);
+  float* Xs = nullptr;
+  gridff_status st = m->fused ? fused_io(m, rows, f, &Xs) : ensure_batch(m, rows);
   if (st != GRIDFF_OK) return st;
   cudaStream_t s = ctx->stream;
   const int Mp = pad16(rows);
   GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->desc, descriptor, n_desc * sizeof(float), cudaMemcpyHostToDevice, s));
-  propose_input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->desc, n_desc, m->sizes[0] - n_desc, rows,
-                                                                         (unsigned long long)seed, Mp, m->pads[0],
-                                                                         m->H[0], m->HT[0]);
-  forward_rows(m, rows);
+  const float* Y = m->fused ? f.Y : m->Y;
+  if (m->fused) fused_forward(m, f, FusedInput{nullptr, m->desc, n_desc, (unsigned long long)seed, 0}, 0);
+  else {
+    propose_input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->desc, n_desc, m->sizes[0] - n_desc, rows,
+                                                                           (unsigned long long)seed, Mp, m->pads[0],
+                                                                           m->H[0], m->HT[0]);
+    forward_rows(m, rows);
+  }
   if (R->rigid) {
-    pose_kernel<<<grid1(rows, 128), 128, 0, s>>>(m->Y, rows, (float)origin_xy[0], (float)origin_xy[1],
+    pose_kernel<<<grid1(rows, 128), 128, 0, s>>>(Y, rows, (float)origin_xy[0], (float)origin_xy[1],
                                                  (float)tile_xy[0], (float)tile_xy[1], R->x);
     GRIDFF_CUDA(ctx, cudaMemsetAsync(R->v, 0, 6 * (size_t)rows * sizeof(float), s));
-  } else if ((st = enqueue_build_poses(R, m->Y, kOut, origin_xy, tile_xy)) != GRIDFF_OK) {
+  } else if ((st = enqueue_build_poses(R, Y, kOut, origin_xy, tile_xy)) != GRIDFF_OK) {
     return st;
   }
   GRIDFF_CUDA(ctx, cudaGetLastError());
