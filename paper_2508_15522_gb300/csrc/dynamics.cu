@@ -2052,14 +2052,22 @@ constexpr int kSwMinBlocks = GRIDFF_SW_MINB;
 #ifndef GRIDFF_RIGID_SUBWARP
 #define GRIDFF_RIGID_SUBWARP -1      // -1: chosen from the molecule size; 0: quad kernel
 #endif
-// Sub-warp width of the rigid relaxation kernel (0 = the quad kernel, used
-// when the cache would not fit): among W = 8, 16, 32 with R = ceil(n / W)
-// atoms per lane, prefer R <= 3 (R = 4 costs registers), then the fewest
-// idle lane slots (n / (W R) largest), then the smaller W.  Measured on
-// GB300 for 10, 24, 38 and 60 atoms this picks the fastest width each time.
+// Sub-warp width of the rigid kernels (0 = the quad kernel, used when the cache
+// would not fit): among W = 8, 16, 32 with R = ceil(n / W) atoms per lane, prefer
+// R <= 3 (R = 4 costs registers), then the fewest idle lane slots (n / (W R)
+// largest), then the smaller W.  Measured on GB300 for 10, 24, 38 and 60 atoms
+// this picks the fastest width of a batch that fills the chip.  A batch that
+// does not (8 warps per SM are resident) takes the widest W that still gives
+// every warp a place: a step's chain is shorter with fewer atoms per lane, and
+// fewer replicas per warp wait for each other's stencil refills.  Where a lane
+// has one atom already, only to half of the places.  us a FIRE step (152 SMs):
+//   10 atoms   64: W8 1.92 W16 1.51 W32 1.41    1001: 1.96 1.55 1.68   2432: 2.06 1.85 3.19
+//   24 atoms   64: W8 2.50 W16 1.85 W32 1.47    1001: 2.83 2.12 1.87   2432: 2.83 2.57 3.41
+//   38 atoms   64:         W16 2.29 W32 1.80    1001:      2.55 2.32   2432:      3.11 4.30
 int rigid_subwarp_width(const gridff_replicas* R) {
   if (GRIDFF_RIGID_SUBWARP >= 0) return GRIDFF_RIGID_SUBWARP;
   const int n = R->max_natoms;
+  auto fits = [&](int W) { return (n + W - 1) / W <= 4 && sw_cache_bytes(n) * kSwWarps * (32 / W) <= 200 * 1024; };
   int best = 0;
   double best_score = -1.0;
   for (int W : {8, 16, 32}) {
@@ -2071,8 +2079,11 @@ int rigid_subwarp_width(const gridff_replicas* R) {
       best = W;
     }
   }
-  if (best == 0) return 0;
-  return sw_cache_bytes(n) * kSwWarps * (32 / best) <= 200 * 1024 ? best : 0;
+  if (best == 0 || !fits(best)) return 0;
+  const long long places = (long long)kSwWarps * kSwMinBlocks * R->ctx->n_sm;
+  for (int W = 32; W > best; W >>= 1)
+    if (fits(W) && ((long long)R->n_rep * W + 31) / 32 <= (n <= W / 2 ? places / 2 : places)) return W;
+  return best;
 }
 
 // Allow `bytes` of dynamic shared memory (needed whenever static plus
