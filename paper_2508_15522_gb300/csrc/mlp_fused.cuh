@@ -88,19 +88,30 @@ __device__ __forceinline__ void ldsm4_t(const void* smem, unsigned (&r)[4]) {
                : "r"((unsigned)__cvta_generic_to_shared(smem)));
 }
 
-// acc[i][c] += A (16 MT rows of sA, k = 0 .. 32 kp - 1) x the n8 tiles
-// w + 8 c (c < 4, below nt) of the fragment-ordered operand B.
-template <int MT>
-__device__ __forceinline__ void rows_gemm(const __nv_bfloat16 (*sA)[kFusedLd], const __nv_bfloat16* __restrict__ B,
-                                          int kp, int nt, int w, int lane, float (&acc)[MT][4][4]) {
-  const int r = (lane & 7) + ((lane >> 3) & 1) * 8, kc = (lane >> 4) * 8;
-  const uint4* b = (const uint4*)B + lane;
-#pragma unroll 4
-  for (int p = 0; p < kp; ++p) {
-    uint4 v[4];
+// A warp's share of a product: the n8 tiles w + 8 c (c < 4, below nt) of the
+// fragment-ordered operand B, k = 0 .. 32 kp - 1.  The whole share of a layer (up
+// to 128 registers) is requested at once and one layer ahead: the weights come
+// from L2, and a load per step of 32 left the kernels waiting (forward 27 us,
+// backward 34 us at 2048 rows; FUSED_MEASURED).
+struct RowsB {
+  uint4 v[4][kFusedW / 32];
+};
+__device__ __forceinline__ void rows_load(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
+  const uint4* b = (const uint4*)W + lane;
+#pragma unroll
+  for (int p = 0; p < kFusedW / 32; ++p)
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (w + 8 * c < nt) v[c] = __ldg(b + ((size_t)(w + 8 * c) * kp + p) * 32);
+      if (p < kp && w + 8 * c < nt) B.v[c][p] = __ldg(b + ((size_t)(w + 8 * c) * kp + p) * 32);
+}
+// acc[i][c] += A (16 MT rows of sA) x B
+template <int MT>
+__device__ __forceinline__ void rows_gemm(const __nv_bfloat16 (*sA)[kFusedLd], const RowsB& B, int kp, int nt, int w,
+                                          int lane, float (&acc)[MT][4][4]) {
+  const int r = (lane & 7) + ((lane >> 3) & 1) * 8, kc = (lane >> 4) * 8;
+#pragma unroll
+  for (int p = 0; p < kFusedW / 32; ++p) {
+    if (p >= kp) break;
 #pragma unroll
     for (int i = 0; i < MT; ++i) {
       unsigned a0[4], a1[4];
@@ -109,8 +120,8 @@ __device__ __forceinline__ void rows_gemm(const __nv_bfloat16 (*sA)[kFusedLd], c
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (w + 8 * c < nt) {
-          mma_bf16(acc[i][c], a0, v[c].x, v[c].y);
-          mma_bf16(acc[i][c], a1, v[c].z, v[c].w);
+          mma_bf16(acc[i][c], a0, B.v[c][p].x, B.v[c][p].y);
+          mma_bf16(acc[i][c], a1, B.v[c][p].z, B.v[c][p].w);
         }
     }
   }
@@ -129,6 +140,8 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
                                       (__nv_bfloat16 (*)[kFusedLd])(smem_h + (size_t)16 * MT * kFusedLd)};
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int m0 = blockIdx.x * 16 * MT;
+  RowsB B;
+  rows_load(B, net.Wf[0], k32(net.pad[0]), net.pad[1] >> 3, w, lane);
   {
     const int ip = net.pad[0], ip32 = 32 * k32(ip), n_in = net.size[0];
     for (int e = tid; e < 16 * MT * ip32; e += 256) {
@@ -155,7 +168,8 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
       for (int c = 0; c < 4; ++c)
 #pragma unroll
         for (int v = 0; v < 4; ++v) acc[i][c][v] = 0.f;
-    rows_gemm<MT>(sH[cur], net.Wf[l], k32(net.pad[l]), nt, w, lane, acc);
+    rows_gemm<MT>(sH[cur], B, k32(net.pad[l]), nt, w, lane, acc);
+    if (!last) rows_load(B, net.Wf[l + 1], k32(op), net.pad[l + 2] >> 3, w, lane);
     const float* bias = net.P + net.boff[l];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -186,8 +200,10 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
   }
 }
 
-// Distance of output o to target t (see gridff.h).
-__device__ __forceinline__ float pose_loss(const FusedLoss& q, const float* o, const float* t, const float* mk) {
+// Distance of output o to target t (see gridff.h), from the torsions'
+// 1 - cos(theta - theta*) in cs.
+__device__ __forceinline__ float pose_loss(const FusedLoss& q, const float* o, const float* t, const float* mk,
+                                           const float* cs) {
   float dx = o[0] - t[0], dy = o[1] - t[1], dz = o[2] - t[2];
   dx -= q.tile_x * rintf(dx / q.tile_x);
   dy -= q.tile_y * rintf(dy / q.tile_y);
@@ -196,7 +212,7 @@ __device__ __forceinline__ float pose_loss(const FusedLoss& q, const float* o, c
   const float s = (o[3] * t[3] + o[4] * t[4] + o[5] * t[5] + o[6] * t[6]) / nu;
   float d = dx * dx + dy * dy + dz * dz + q.w_q * (1.f - s * s);
   if (mk)
-    for (int j = 0; j < 12; ++j) d += q.w_t * mk[j] * (1.f - cosf(o[7 + j] - t[7 + j]));
+    for (int j = 0; j < 12; ++j) d += q.w_t * mk[j] * cs[j];
   return d;
 }
 
@@ -209,20 +225,31 @@ __device__ __forceinline__ int target_row(const FusedLoss& q, int b) {
 // regard to the proposals per target; the block with a target's first row
 // writes its loss.  Writes dL/da of every layer in FP32 (bias gradients) and
 // as the bfloat16 operand (weight gradients).
-constexpr int kLossMax = 512;       // proposals evaluated per block at most: K <= 240
+constexpr int kLossMax = 512;       // proposals evaluated per block at most: K <= 248
+constexpr int kLossTargets = 20;    // targets per block at most (K = 1: 16)
 __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, FusedLoss q) {
   __shared__ __align__(16) __nv_bfloat16 sG[2][16][kFusedLd];
-  __shared__ float s_d[kLossMax];
-  __shared__ int s_win[20];
+  __shared__ float s_cos[kLossMax * 12], s_d[kLossMax];
+  __shared__ int s_row[kLossTargets], s_win[kLossTargets];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int m0 = blockIdx.x * 16, L = net.L, K = q.K, n_out = net.size[L], opl = net.pad[L];
   const int ba = m0 / K, bb = min(q.n_targets - 1, (m0 + 15) / K), nb = bb - ba + 1;
-  for (int e = tid; e < nb * K; e += 256) {
-    const int b = ba + e / K, row = target_row(q, b);
-    s_d[e] = pose_loss(q, net.Y + ((size_t)ba * K + e) * n_out, q.T + (size_t)row * 19,
-                       q.mask ? q.mask + (size_t)row * 12 : nullptr);
-  }
+  RowsB B;
+  if (L > 1) rows_load(B, net.Wr[L - 1], k32(opl), net.pad[L - 1] >> 3, w, lane);
+  if (tid < nb) s_row[tid] = target_row(q, ba + tid);
   for (int e = tid; e < 16 * 32 * k32(opl); e += 256) sG[0][e / (32 * k32(opl))][e % (32 * k32(opl))] = __float2bfloat16(0.f);
+  __syncthreads();
+  const float* Yb = net.Y + (size_t)ba * K * n_out;
+  if (q.mask)
+    for (int e = tid; e < nb * K * 12; e += 256) {
+      const int p = e / 12, j = e % 12;
+      s_cos[e] = 1.f - cosf(Yb[(size_t)p * n_out + 7 + j] - q.T[(size_t)s_row[p / K] * 19 + 7 + j]);
+    }
+  __syncthreads();
+  for (int e = tid; e < nb * K; e += 256) {
+    const size_t row = s_row[e / K];
+    s_d[e] = pose_loss(q, Yb + (size_t)e * n_out, q.T + row * 19, q.mask ? q.mask + row * 12 : nullptr, s_cos + 12 * e);
+  }
   __syncthreads();
   if (tid < nb) {
     const int b = ba + tid;
@@ -247,7 +274,7 @@ __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, Fused
     float g = 0.f;
     const int b = m / K;
     if (m < net.rows && j < n_out && s_win[b - ba] == m) {
-      const int row = target_row(q, b);
+      const int row = s_row[b - ba];
       const float *o = net.Y + (size_t)m * n_out, *t = q.T + (size_t)row * 19;
       const float* mk = q.mask ? q.mask + (size_t)row * 12 : nullptr;
       const float inv_b = 1.f / q.n_targets;
@@ -280,7 +307,8 @@ __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, Fused
     for (int c = 0; c < 4; ++c)
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[0][c][v] = 0.f;
-    rows_gemm<1>(sG[cur], net.Wr[l], k32(net.pad[l + 1]), nt, w, lane, acc);
+    rows_gemm<1>(sG[cur], B, k32(net.pad[l + 1]), nt, w, lane, acc);
+    if (l > 1) rows_load(B, net.Wr[l - 1], k32(ip), net.pad[l - 1] >> 3, w, lane);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (w + 8 * c >= nt) continue;
