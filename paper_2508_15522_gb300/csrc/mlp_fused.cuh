@@ -92,39 +92,52 @@ __device__ __forceinline__ void ldsm4_t(const void* smem, unsigned (&r)[4]) {
 // fragment-ordered operand B, k = 0 .. 32 kp - 1.  The whole share of a layer (up
 // to 128 registers) is requested at once and one layer ahead: the weights come
 // from L2, and a load per step of 32 left the kernels waiting (forward 27 us,
-// backward 34 us at 2048 rows; FUSED_MEASURED).
+// backward 34 us at 2048 rows, now 14 and 20).
 struct RowsB {
   uint4 v[4][kFusedW / 32];
 };
-__device__ __forceinline__ void rows_load(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
+// FULL: 256 inputs and 256 outputs, no tile of the share is missing.
+template <bool FULL>
+__device__ __forceinline__ void rows_load_t(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
   const uint4* b = (const uint4*)W + lane;
 #pragma unroll
   for (int p = 0; p < kFusedW / 32; ++p)
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (p < kp && w + 8 * c < nt) B.v[c][p] = __ldg(b + ((size_t)(w + 8 * c) * kp + p) * 32);
+      if (FULL || (p < kp && w + 8 * c < nt)) B.v[c][p] = __ldg(b + ((w + 8 * c) * (FULL ? kFusedW / 32 : kp) + p) * 32);
+}
+__device__ __forceinline__ bool rows_full(int kp, int nt) { return kp == kFusedW / 32 && nt == kFusedW / 8; }
+__device__ __forceinline__ void rows_load(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
+  if (rows_full(kp, nt)) rows_load_t<true>(B, W, kp, nt, w, lane);
+  else rows_load_t<false>(B, W, kp, nt, w, lane);
 }
 // acc[i][c] += A (16 MT rows of sA) x B
-template <int MT>
-__device__ __forceinline__ void rows_gemm(const __nv_bfloat16 (*sA)[kFusedLd], const RowsB& B, int kp, int nt, int w,
-                                          int lane, float (&acc)[MT][4][4]) {
-  const int r = (lane & 7) + ((lane >> 3) & 1) * 8, kc = (lane >> 4) * 8;
+template <int MT, bool FULL>
+__device__ __forceinline__ void rows_gemm_t(const __nv_bfloat16 (*sA)[kFusedLd], const RowsB& B, int kp, int nt, int w,
+                                            int lane, float (&acc)[MT][4][4]) {
+  const __nv_bfloat16* a = &sA[(lane & 7) + ((lane >> 3) & 1) * 8][(lane >> 4) * 8];
 #pragma unroll
   for (int p = 0; p < kFusedW / 32; ++p) {
-    if (p >= kp) break;
+    if (!FULL && p >= kp) break;
 #pragma unroll
     for (int i = 0; i < MT; ++i) {
       unsigned a0[4], a1[4];
-      ldsm4(&sA[16 * i + r][32 * p + kc], a0);
-      ldsm4(&sA[16 * i + r][32 * p + 16 + kc], a1);
+      ldsm4(a + 16 * i * kFusedLd + 32 * p, a0);
+      ldsm4(a + 16 * i * kFusedLd + 32 * p + 16, a1);
 #pragma unroll
       for (int c = 0; c < 4; ++c)
-        if (w + 8 * c < nt) {
-          mma_bf16(acc[i][c], a0, B.v[c][p].x, B.v[c][p].y);
-          mma_bf16(acc[i][c], a1, B.v[c][p].z, B.v[c][p].w);
-        }
+        if (FULL || w + 8 * c < nt) mma_bf16(acc[i][c], a0, B.v[c][p].x, B.v[c][p].y);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (FULL || w + 8 * c < nt) mma_bf16(acc[i][c], a1, B.v[c][p].z, B.v[c][p].w);
     }
   }
+}
+template <int MT>
+__device__ __forceinline__ void rows_gemm(const __nv_bfloat16 (*sA)[kFusedLd], const RowsB& B, int kp, int nt, int w,
+                                          int lane, float (&acc)[MT][4][4]) {
+  if (rows_full(kp, nt)) rows_gemm_t<MT, true>(sA, B, kp, nt, w, lane, acc);
+  else rows_gemm_t<MT, false>(sA, B, kp, nt, w, lane, acc);
 }
 
 // Forward of 16 MT rows per block of 8 warps, all layers; every warp has the
@@ -144,18 +157,21 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
   rows_load(B, net.Wf[0], k32(net.pad[0]), net.pad[1] >> 3, w, lane);
   {
     const int ip = net.pad[0], ip32 = 32 * k32(ip), n_in = net.size[0];
-    for (int e = tid; e < 16 * MT * ip32; e += 256) {
-      const int r = e / ip32, k = e % ip32, m = m0 + r;
-      float v = 0.f;
-      if (m < net.rows && k < n_in) {
-        if (in.X) v = in.X[(size_t)m * n_in + k];
-        else if (k < in.n_desc) v = in.desc[k];
-        else v = normal_of(splitmix64(in.seed ^ splitmix64(((in.base + (unsigned long long)m) << 6) + (k - in.n_desc))));
+    // 16 threads a row, columns 16 apart: the noise inputs (a logarithm, a square
+    // root and a cosine) fall to all threads alike
+    for (int r = tid >> 4; r < 16 * MT; r += 16)
+      for (int k = tid & 15; k < ip32; k += 16) {
+        const int m = m0 + r;
+        float v = 0.f;
+        if (m < net.rows && k < n_in) {
+          if (in.X) v = in.X[(size_t)m * n_in + k];
+          else if (k < in.n_desc) v = in.desc[k];
+          else v = normal_of(splitmix64(in.seed ^ splitmix64(((in.base + (unsigned long long)m) << 6) + (k - in.n_desc))));
+        }
+        const __nv_bfloat16 b = __float2bfloat16(v);
+        sH[0][r][k] = b;
+        if (train && k < ip && m < net.Mp) net.H[0][(size_t)m * ip + k] = b;
       }
-      const __nv_bfloat16 b = __float2bfloat16(v);
-      sH[0][r][k] = b;
-      if (train && k < ip && m < net.Mp) net.H[0][(size_t)m * ip + k] = b;
-    }
   }
   __syncthreads();
   for (int l = 0; l < net.L; ++l) {
@@ -307,6 +323,16 @@ __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, Fused
     for (int c = 0; c < 4; ++c)
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[0][c][v] = 0.f;
+    // the layer's activations (their sign is the mask), requested before the product
+    __nv_bfloat162 act[4][2];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int m = m0 + (lane >> 2) + 8 * h;
+        if (w + 8 * c < nt && m < net.rows)
+          act[c][h] = *(const __nv_bfloat162*)&net.H[l][(size_t)m * ip + 8 * (w + 8 * c) + 2 * (lane & 3)];
+      }
     rows_gemm<1>(sG[cur], B, k32(net.pad[l + 1]), nt, w, lane, acc);
     if (l > 1) rows_load(B, net.Wr[l - 1], k32(ip), net.pad[l - 1] >> 3, w, lane);
 #pragma unroll
@@ -318,7 +344,7 @@ __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, Fused
         const int r = (lane >> 2) + 8 * h, m = m0 + r;
         float2 v = make_float2(0.f, 0.f);
         if (m < net.rows) {
-          const float2 a = __bfloat1622float2(*(const __nv_bfloat162*)&net.H[l][(size_t)m * ip + j]);
+          const float2 a = __bfloat1622float2(act[c][h]);
           if (j < n_in && a.x > 0.f) v.x = acc[0][c][2 * h];
           if (j + 1 < n_in && a.y > 0.f) v.y = acc[0][c][2 * h + 1];
         }
