@@ -9,6 +9,7 @@
 // scattered 16-byte pieces; the quad then sums its partial contractions with
 // two shuffles.  Flexible replicas keep positions, velocities and forces in
 // shared memory; the integrator updates run with lanes over atoms.
+#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -1034,14 +1035,14 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// The hand-off flag's value once it is set, or 0 when the bounded wait ran
-// out (one lane calls it).
-__device__ __noinline__ int wait_handoff(const int* flag) {
+// The hand-off flag's value once it counts `parts` ended parts (bits 0 .. 15),
+// or its last value when the bounded wait ran out (one lane calls it).
+__device__ __noinline__ int wait_handoff(const int* flag, int parts) {
   const unsigned long long deadline = gtimer() + kHandoffWaitNs;
   int hv = 0;
   for (int k = 0; k < kHandoffPolls; ++k) {
     hv = ld_acquire(flag);
-    if (hv != 0 || gtimer() > deadline) break;
+    if ((hv & 0xffff) >= parts || gtimer() > deadline) break;
     __nanosleep(1000);
   }
   return hv;
@@ -1068,34 +1069,49 @@ relax_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_t
   const int n_warps = gridDim.x * WPB;
   const unsigned long long t0 = gtimer();
   // Relaxations that may stop early (f_conv > 0) have unknown lengths:
-  // there the warps take whole tasks from an atomic queue (greedy list
-  // scheduling) instead of the time-sliced ranges.
+  // there the warps take tasks from an atomic queue instead of the
+  // time-sliced ranges, in `queued` parts of equal iteration ranges, every
+  // task's first part before any second one (sw_queue_parts).  A part begins
+  // when the task's part before it has ended.
   const int n_tasks = (n_rep + RPW - 1) / RPW;
   for (int j = 0;; ++j) {      // uniform over the warp
     SwPart part;
+    int after = 0;            // parts of the task that must have ended before
+    bool hands_on = false;    // a later part of the task follows
     if (queued) {
       int next = 0;
       if (lane == 0) next = atomicAdd(&ctl.res->next, 1);
       next = __shfl_sync(kFull, next, 0);
-      part = SwPart{next < n_tasks ? next : -1, 0, nsteps, 0};
+      const int c = next / n_tasks;
+      part = SwPart{c < queued ? next - c * n_tasks : -1, (int)((long long)nsteps * c / queued),
+                    (int)((long long)nsteps * (c + 1) / queued), 0};
+      after = c;
+      hands_on = c + 1 < queued;
     } else {
       part = sw_part(warp, n_warps, n_tasks, nsteps, j);
     }
     if (part.p < 0) break;
     const int p = part.p, it_b = part.it_b, it_e = part.it_e;
-    const bool head = part.role == 1, tail = part.role == 2;
-    // flag value of a finished head: bit 0 set, bit 1 + s set when the
-    // abort flag or the clock budget stopped replica s of the task
-    int hv = 1;
-    if (tail) {
-      // wait until the previous warp has written the head of this task
+    if (!queued) {
+      after = part.role == 2;
+      hands_on = part.role == 1;
+    }
+    const bool head = hands_on;
+    // a task's flag: bits 0 .. 15 the parts that have ended, bit 16 + s set
+    // when the abort flag or the clock budget stopped replica s of the task
+    int hv = 0;
+    if (after > 0) {
+      // wait until another warp has written the parts before
       if (lane == 0) {
-        hv = wait_handoff(handoff + p);
-        if (hv == 0) atomicAdd(&ctl.res->handoff_timeouts, 1);
+        hv = wait_handoff(handoff + p, after);
+        if ((hv & 0xffff) < after) {
+          atomicAdd(&ctl.res->handoff_timeouts, 1);
+          hv = -1;
+        }
       }
       hv = __shfl_sync(kFull, hv, 0);
       __syncwarp();
-      if (hv == 0) continue;
+      if (hv < 0) continue;
     }
     const int r = p * RPW + sw;
     const bool valid = r < n_rep;
@@ -1142,8 +1158,8 @@ relax_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_t
     const float ang_cap = fp.d_max / rmax;
     float elane = 0.f;
     // a tail whose head was stopped stops too (the head's state is final)
-    bool done = !valid || ((hv >> (1 + sw)) & 1);
-    bool stopped = false;
+    bool done = !valid || ((hv >> (16 + sw)) & 1);
+    bool stopped = valid && done;
     for (int it = it_b; it < it_e; ++it) {
       if ((it & 31) == 0) {
         int sb = 0;
@@ -1255,14 +1271,14 @@ relax_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_t
       report(ctl, n, evals, head ? (st & ~GRIDFF_REP_CONVERGED) : st, total);
     }
     if (head && publish) {
-      // publish the head's state to the warp that runs the tail
+      // publish this part's state to the warp that runs the next one
       const unsigned sm = __ballot_sync(kFull, stopped && l == 0);
       __threadfence();
       __syncwarp();
       if (lane == 0) {
-        int v = 1;
+        int v = after + 1;
         for (int s2 = 0; s2 < RPW; ++s2)
-          if ((sm >> (s2 * W)) & 1u) v |= 2 << s2;
+          if ((sm >> (s2 * W)) & 1u) v |= 0x10000 << s2;
         st_release(handoff + p, v);
       }
     }
@@ -1857,7 +1873,7 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
     int hv = 1;
     if (tail) {
       if (lane == 0) {
-        hv = wait_handoff(handoff + part.p);
+        hv = wait_handoff(handoff + part.p, 1);
         if (hv == 0) atomicAdd(&ctl.res->handoff_timeouts, 1);
       }
       hv = __shfl_sync(kFull, hv, 0);
@@ -1866,7 +1882,7 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
     }
     const int r = part.p * RPW + sw;
     // a replica whose head was stopped keeps the head's final state
-    const bool valid = r < n_rep && !((hv >> (1 + sw)) & 1);
+    const bool valid = r < n_rep && !((hv >> (16 + sw)) & 1);
     int n = 0, ab = 0;
     float4 rig = make_float4(1.f, 1.f, 1.f, 1.f);
     float c[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, v[3] = {0.f, 0.f, 0.f}, p[4] = {0.f, 0.f, 0.f, 0.f};
@@ -2006,7 +2022,7 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
       if (lane == 0) {
         int hvv = 1;
         for (int s2 = 0; s2 < RPW; ++s2)
-          if ((sm >> (s2 * W)) & 1u) hvv |= 2 << s2;
+          if ((sm >> (s2 * W)) & 1u) hvv |= 0x10000 << s2;
         st_release(handoff + part.p, hvv);
       }
     }
@@ -2391,6 +2407,29 @@ cudaError_t launch_ex(void (*fn)(KArgs...), int blocks, int threads, size_t dyn,
 
 }  // namespace
 
+// Parts per task of the rigid queue.  Whole tasks leave warps idle in the last
+// round (4096 replicas of 38 atoms: 2048 tasks on 1216 warps take 2 rounds for
+// 1.68 of work); with C parts per task the rounds are ceil(C tasks / warps) / C.
+// A part costs about one and a half iterations more (its state through L2, every
+// stencil of its atoms refilled), so C minimises the sum.  Parts are at most 4096
+// iterations (0.2 s of the largest molecules), well inside the bounded wait.
+// 4096 x 38 atoms, 200 iterations a call: 1189 -> 1073 us (4 parts).
+static int sw_queue_parts(long long tasks, long long warps, int nsteps) {
+  if (tasks <= warps) return 1;
+  const int least = std::max(2, (nsteps + 4095) / 4096);
+  const long long most = std::min<long long>(std::max(least, 64), std::min<long long>(0xffff, (1LL << 30) / tasks));
+  int best = 1;
+  double best_cost = (double)((tasks + warps - 1) / warps) * nsteps;
+  for (int C = least; C <= most && nsteps / C >= 32; ++C) {
+    const double cost = (double)((tasks * C + warps - 1) / warps) / C * (nsteps + 1.5 * C);
+    if (cost < best_cost * (1 - 1e-9)) {
+      best_cost = cost;
+      best = C;
+    }
+  }
+  return best;
+}
+
 gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, const LaunchCfg& c,
                             int blocks, int nsteps, const gridff_fire_params& P, int flags) {
   cudaStream_t s = ctx->stream;
@@ -2435,7 +2474,10 @@ gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
       e = launch_ex(rigid_sw_fn(c.W, sw_rounds(R, c.W), kind), blocks, k.threads, k.dyn, s, wp, gv, R->tv,
                     (const int*)R->rep_tmpl, R->n_rep, R->x, R->v, R->fire_dt, R->fire_alpha, R->fire_nplus,
                     R->status, R->steps, R->energy, R->last_x, R->last_f, R->handoff,
-                    (int)(c.queue == 1 || (c.queue == 0 && P.f_conv > 0)), (int)!(flags & GRIDFF_TEST_NO_HANDOFF),
+                    c.queue == 1 || (c.queue == 0 && P.f_conv > 0)
+                        ? sw_queue_parts((R->n_rep + 32 / c.W - 1) / (32 / c.W), kSwWarps * blocks, nsteps)
+                        : 0,
+                    (int)!(flags & GRIDFF_TEST_NO_HANDOFF),
                     nsteps, fp, ctl, c.S);
       break;
     case GRIDFF_KERNEL_RIGID_QUAD:
