@@ -48,9 +48,12 @@ __device__ __forceinline__ void store_eg(WarpState& s, int i, float e) { s.eg[i]
 __device__ __forceinline__ void store_eg(WarpStateEval& s, int i, float e) { s.eg[i] = e; }
 __device__ __forceinline__ void store_eg(WarpStateXF&, int, float) {}
 
-// Bytes of one replica's share in the sub-warp kernels: its stencil cache
-// and the cells its lanes publish for the refill queue (int2 per slot).
-__host__ __device__ constexpr size_t sw_cache_bytes(int S) { return cache_bytes(S) + (((size_t)S * 8 + 15) & ~size_t(15)); }
+// Bytes of one replica's stencil cache in the sub-warp kernels, and of one warp:
+// its replicas' caches and the list of stencils to refill (int2 per atom).
+__host__ __device__ constexpr size_t sw_cache_bytes(int S) { return cache_bytes(S); }
+__host__ __device__ constexpr size_t sw_warp_bytes(int S, int rpw) {
+  return (size_t)rpw * sw_cache_bytes(S) + (((size_t)rpw * S * 8 + 15) & ~size_t(15));
+}
 
 // Bytes of one warp's dynamic shared memory in the unique-term flexible
 // kernel: its stencil cache and the staged nonbonded parameters.
@@ -811,10 +814,12 @@ relax_rigid_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl
 // body-frame torque summed over the sub-warp, this lane's share of the
 // energy (Acc: float for relaxations, double for NVE) and the BELOW flag.
 template <int W, int R, int KIND, class Acc>
-__device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache& sc, float* cval, int2* pub,
-                                          const float4* __restrict__ par, int S, int sw, int l, int n, bool run,
+__device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache& sc, unsigned char* wval, int2* list,
+                                          const float4* __restrict__ par, int ab, int S, int lane, int sw, int l, int n,
+                                          bool run,
                                           const float c[3], const float Rm[9], const float4 (&bk)[R],
                                           const float4 (&pk)[R], float Ft[3], float tq[3], Acc& e, int& flags) {
+  const size_t stride = sw_cache_bytes(S);     // from one replica's cache to the next
   for (int a = 0; a < 3; ++a) Ft[a] = tq[a] = 0.f;
   e = Acc(0);
   // locate every atom of the lane
@@ -833,46 +838,43 @@ __device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache&
     cl[k] = locate(g, act, px, py, pz, flags);
     key[k] = (cl[k].ix * g.ny + cl[k].iy) * g.nz + cl[k].iz;
     const bool miss = cl[k].inside && sc.key[i < S ? i : 0] != key[k];
-    unsigned msub = __ballot_sync(kFull, miss);
-    if constexpr (W < 32) msub = (msub >> (sw * W)) & ((1u << (W & 31)) - 1u);
-    miss_mask[k] = msub;
+    miss_mask[k] = __ballot_sync(kFull, miss);
   }
-  // refill the stencils that changed cell.  Each lane publishes the cells
-  // of its atoms that missed; the misses of all rounds k form one queue
-  // (bit k W + l = atom index), served W/4 atoms at a time (one per quad)
-  // with one copy of the gather code
+  // Refill the stencils that changed cell.  All misses of the warp, whichever
+  // of its replicas they belong to, form one list in shared memory (record of
+  // the stencil's first node, atom slot and sub-warp; an entry's rank from the
+  // ballots), which the warp's eight quads serve eight at a time: a gather is an L2 round
+  // trip, so what counts is how many follow each other.
+  {
+    int total = 0;
 #pragma unroll
-  for (int k = 0; k < R; ++k)
-    if ((miss_mask[k] >> l) & 1u) pub[k * W + l] = make_int2(cl[k].ix | (cl[k].iy << 16), cl[k].iz);
-  __syncwarp();
-  constexpr int kPerWord = 64 / W;   // rounds k whose miss bits share one 64-bit word
-#pragma unroll
-  for (int k0 = 0; k0 < R; k0 += kPerWord) {
-    unsigned long long mm = 0;
-#pragma unroll
-    for (int k = k0; k < R && k < k0 + kPerWord; ++k) mm |= (unsigned long long)miss_mask[k] << ((k - k0) * W);
-#pragma unroll 1
-    while (__any_sync(kFull, mm != 0)) {
-      const int qd = l >> 2, qq = l & 3;
-      unsigned long long m = mm;
-      for (int j = 0; j < qd && m; ++j) m &= m - 1;
-      if (m) {
-        const int slot = k0 * W + __ffsll((long long)m) - 1;
-        const int2 pc = pub[slot];
-        const int oix = (int)((unsigned)pc.x & 0xffffu), oiy = (int)((unsigned)pc.x >> 16), oiz = pc.y;
-        float cv[16];
-        gather_runs<KIND>(g, ((long long)oix * g.nyp + oiy) * g.nzp + oiz + qq, __ldg(&par[slot]), cv);
-        // run mm = 4a + b, z-node qq goes to float4 2p + (qq >> 1) of
-        // run pair p = 2a + (b >> 1), component 2 (qq & 1) + (b & 1)
-#pragma unroll
-        for (int r2 = 0; r2 < 16; ++r2) {
-          const int a = r2 >> 2, bq = r2 & 3;
-          const int f4 = 2 * (2 * a + (bq >> 1)) + (qq >> 1);
-          cval[((size_t)f4 * S + slot) * 4 + 2 * (qq & 1) + (bq & 1)] = cv[r2];
-        }
-        if (qq == 0) sc.key[slot] = (oix * g.ny + oiy) * g.nz + oiz;
+    for (int k = 0; k < R; ++k) {
+      const unsigned bal = miss_mask[k];
+      if ((bal >> lane) & 1u) {
+        const int slot = k * W + l;
+        list[total + __popc(bal & ((1u << lane) - 1u))] =
+            make_int2((int)(unsigned)(((long long)cl[k].ix * g.nyp + cl[k].iy) * g.nzp + cl[k].iz), slot | (sw << 8));
+        sc.key[slot] = key[k];
       }
-      for (int j = 0; j < W / 4 && mm; ++j) mm &= mm - 1;
+      total += __popc(bal);
+    }
+    __syncwarp();
+    const int qd = lane >> 2, qq = lane & 3;
+#pragma unroll 1
+    for (int j = 0; j < total; j += kQuads) {
+      const bool on = j + qd < total;
+      const int2 e = list[on ? j + qd : 0];
+      const int s2 = e.y >> 8, slot = e.y & 0xff;
+      const int a = __shfl_sync(kFull, ab, s2 * W);      // the entry's template: its replica's
+      if (on) {
+        float cv[16];
+        gather_runs<KIND>(g, (long long)(unsigned)e.x + qq, __ldg(&par[a + slot]), cv);
+        // runs (a, b) and (a, b + 1), b even, z-node qq go to float4 2p +
+        // (qq >> 1) of run pair p = 2a + (b >> 1), half qq & 1: one 8-byte store
+        float2* const dst = (float2*)(wval + (size_t)s2 * stride) + 2 * ((qq >> 1) * S + slot) + (qq & 1);
+#pragma unroll
+        for (int p = 0; p < 8; ++p) dst[4 * p * S] = make_float2(cv[2 * p], cv[2 * p + 1]);
+      }
     }
   }
   __syncwarp();
@@ -1058,13 +1060,13 @@ relax_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_t
   constexpr int RPW = 32 / W;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int sw = lane / W, l = lane % W;
-  unsigned char* const wbase = dyn_smem + (size_t)(wib * RPW + sw) * sw_cache_bytes(S);
+  // the warp's replicas' caches (stencils, keys), then its refill list
+  unsigned char* const wval = dyn_smem + (size_t)wib * sw_warp_bytes(S, RPW);
+  int2* const list = (int2*)(wval + (size_t)RPW * sw_cache_bytes(S));
   StencilCache sc;
-  sc.val = (float4*)wbase;
-  sc.key = (int*)(wbase + (size_t)S * 256);
+  sc.val = (float4*)(wval + (size_t)sw * sw_cache_bytes(S));
+  sc.key = (int*)((unsigned char*)sc.val + (size_t)S * 256);
   sc.S = S;
-  int2* const pub = (int2*)(wbase + cache_bytes(S));
-  float* const cval = (float*)sc.val;
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
   const unsigned long long t0 = gtimer();
@@ -1182,7 +1184,7 @@ relax_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_t
       float Ft[3], tq[3];
       float e = 0.f;
       int flags = 0;
-      sw_forces<W, R, KIND, float>(g, sc, cval, pub, tv.par + ab, S, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
+      sw_forces<W, R, KIND, float>(g, sc, wval, list, tv.par, ab, S, lane, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
                                     flags);
       if (!run) continue;
       st |= flags;
@@ -1853,13 +1855,13 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
   constexpr int RPW = 32 / W;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int sw = lane / W, l = lane % W;
-  unsigned char* const wbase = dyn_smem + (size_t)(wib * RPW + sw) * sw_cache_bytes(S);
+  // the warp's replicas' caches (stencils, keys), then its refill list
+  unsigned char* const wval = dyn_smem + (size_t)wib * sw_warp_bytes(S, RPW);
+  int2* const list = (int2*)(wval + (size_t)RPW * sw_cache_bytes(S));
   StencilCache sc;
-  sc.val = (float4*)wbase;
-  sc.key = (int*)(wbase + (size_t)S * 256);
+  sc.val = (float4*)(wval + (size_t)sw * sw_cache_bytes(S));
+  sc.key = (int*)((unsigned char*)sc.val + (size_t)S * 256);
   sc.S = S;
-  int2* const pub = (int2*)(wbase + cache_bytes(S));
-  float* const cval = (float*)sc.val;
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
   const unsigned long long t0 = gtimer();
@@ -1949,7 +1951,7 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
     bool run = valid, stopped = false;
     // forces at the start of the part (a tail recomputes those its head
     // ended with: the same values)
-    sw_forces<W, R, KIND, double>(g, sc, cval, pub, tv.par + ab, S, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
+    sw_forces<W, R, KIND, double>(g, sc, wval, list, tv.par, ab, S, lane, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
                                   flags);
     if (it_b == 0) {
       const double e0 = sub_sum(e);
@@ -1984,7 +1986,7 @@ run_rigid_sw_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmp
       }
       quat_rot(q[0], q[1], q[2], q[3], Rm);
       int f2 = 0;
-      sw_forces<W, R, KIND, double>(g, sc, cval, pub, tv.par + ab, S, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
+      sw_forces<W, R, KIND, double>(g, sc, wval, list, tv.par, ab, S, lane, sw, l, n, run, c, Rm, bk, pk, Ft, tq, e,
                                     f2);
       if (run) {
         flags |= f2;
@@ -2083,7 +2085,7 @@ constexpr int kSwMinBlocks = GRIDFF_SW_MINB;
 int rigid_subwarp_width(const gridff_replicas* R) {
   if (GRIDFF_RIGID_SUBWARP >= 0) return GRIDFF_RIGID_SUBWARP;
   const int n = R->max_natoms;
-  auto fits = [&](int W) { return (n + W - 1) / W <= 4 && sw_cache_bytes(n) * kSwWarps * (32 / W) <= 200 * 1024; };
+  auto fits = [&](int W) { return (n + W - 1) / W <= 4 && sw_warp_bytes(n, 32 / W) * kSwWarps <= 200 * 1024; };
   int best = 0;
   double best_score = -1.0;
   for (int W : {8, 16, 32}) {
@@ -2206,7 +2208,7 @@ KernelShape shape_of(const gridff_replicas* R, const LaunchCfg& c, int kind) {
       if (!R->rigid || (c.W != 8 && c.W != 16 && c.W != 32) || c.S < R->max_natoms) return k;
       const SwFn fn = rigid_sw_fn(c.W, sw_rounds(R, c.W), kind);
       if (!fn) return k;
-      return {(const void*)fn, 32 * kSwWarps, kSwWarps * (32 / c.W), sw_cache_bytes(c.S) * kSwWarps * (32 / c.W)};
+      return {(const void*)fn, 32 * kSwWarps, kSwWarps * (32 / c.W), sw_warp_bytes(c.S, 32 / c.W) * kSwWarps};
     }
     case GRIDFF_KERNEL_RIGID_QUAD:
       if (!R->rigid || c.wpb != kWarpsPerBlock) return k;
@@ -2710,7 +2712,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
     if (fn) {
       // the sub-warp layout of the relaxation, every atom cached
       const int S = R->max_natoms;
-      const size_t dyn = sw_cache_bytes(S) * kSwWarps * (32 / W);
+      const size_t dyn = sw_warp_bytes(S, 32 / W) * kSwWarps;
       GRIDFF_CUDA(ctx, set_dyn_smem((const void*)fn, dyn));
       const int per_block = kSwWarps * (32 / W);
       int per_sm = 0;
