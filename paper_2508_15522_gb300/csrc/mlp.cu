@@ -659,7 +659,24 @@ gridff_status fused_workspace(gridff_mlp* m, int rows, FusedNet& f, FusedLoss& q
   return GRIDFF_OK;
 }
 
-void fused_forward(gridff_mlp* m, const FusedNet& f, const FusedInput& in, int train) {
+// Launch of one of a step's kernels; `ahead`: it may start while the launch
+// before it, another of them, is at work (previous_done()).
+template <class... P, class... A>
+void fused_launch(gridff_mlp* m, void (*fn)(P...), int blocks, int threads, size_t dyn, bool ahead, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = m->ctx->stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = ahead ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, fn, P(args)...);      // errors: cudaGetLastError() of the caller
+}
+
+void fused_forward(gridff_mlp* m, const FusedNet& f, const FusedInput& in, int train, bool ahead) {
   // 64 rows a block re-read the weights a quarter as often and need enough
   // rows for the chip
   const bool wide = f.rows >= 8192;
@@ -667,16 +684,15 @@ void fused_forward(gridff_mlp* m, const FusedNet& f, const FusedInput& in, int t
   const size_t dyn = 2 * (size_t)per * kFusedLd * sizeof(__nv_bfloat16);
   auto fn = wide ? fused_forward_kernel<4> : fused_forward_kernel<1>;
   if (wide) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  fn<<<(f.Mp + per - 1) / per, 256, dyn, m->ctx->stream>>>(f, in, train);
+  fused_launch(m, fn, (f.Mp + per - 1) / per, 256, dyn, ahead, f, in, train);
 }
 
 // One training step: forward, loss and backward, gradients, update; hist: slot
 // of the step's mean loss, or null.  Enqueued, no synchronisation.
 gridff_status fused_step(gridff_mlp* m, const FusedNet& f, const FusedInput& in, const FusedLoss& q,
-                         const gridff_train_params* tp, long long t, int update, float* hist) {
-  cudaStream_t s = m->ctx->stream;
-  fused_forward(m, f, in, 1);
-  fused_backward_kernel<<<f.Mp / 16, 256, 0, s>>>(f, q);
+                         const gridff_train_params* tp, long long t, int update, float* hist, bool ahead) {
+  fused_forward(m, f, in, 1, ahead);
+  fused_launch(m, fused_backward_kernel, f.Mp / 16, 256, 0, true, f, q);
   GradMap g{};
   int n = 0;
   for (int l = 0; l < f.L; ++l) {
@@ -691,13 +707,14 @@ gridff_status fused_step(gridff_mlp* m, const FusedNet& f, const FusedInput& in,
     n += (f.size[l + 1] + 31) / 32 * f.chunks;
   }
   g.db_first[f.L] = n - g.first[f.L];
-  fused_grad_kernel<<<n, 128, 0, s>>>(f, g);
+  fused_launch(m, fused_grad_kernel, n, 128, 0, true, f, g);
   AdamArgs ad{tp->beta1, tp->beta2, tp->eps, 0.f, 0.f, update};
   if (update) {
     ad.c1 = (float)(tp->lr / (1.0 - pow((double)tp->beta1, (double)t)));
     ad.c2 = (float)(1.0 / (1.0 - pow((double)tp->beta2, (double)t)));
   }
-  fused_update_kernel<<<grid1((long long)m->n_params) + 1, 256, 0, s>>>(f, ad, (int)m->n_params, q.loss, q.n_targets, hist);
+  fused_launch(m, fused_update_kernel, grid1((long long)m->n_params) + 1, 256, 0, true, f, ad, (int)m->n_params, q.loss,
+               q.n_targets, hist);
   GRIDFF_CUDA(m->ctx, cudaGetLastError());
   return GRIDFF_OK;
 }
@@ -905,7 +922,7 @@ gridff_status gridff_mlp_forward(gridff_mlp* m, int32_t rows, const float* x, fl
     const gridff_status fs = fused_io(m, rows, f, &Xs);
     if (fs != GRIDFF_OK) return fs;
     GRIDFF_CUDA(ctx, cudaMemcpyAsync(Xs, x, (size_t)rows * m->sizes[0] * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
-    fused_forward(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, 0);
+    fused_forward(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, 0, false);
     GRIDFF_CUDA(ctx, cudaGetLastError());
     GRIDFF_CUDA(ctx, cudaMemcpyAsync(y, f.Y, (size_t)rows * kOut * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
     GRIDFF_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -964,7 +981,8 @@ gridff_status gridff_mlp_train_step(gridff_mlp* m, int32_t n_targets, int32_t K,
     q.tile_y = (float)tp->tile[1];
     const int update = !(flags & GRIDFF_MLP_NO_UPDATE);
     m->t += update;
-    if ((st = fused_step(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, q, tp, m->t, update, nullptr)) != GRIDFF_OK) return st;
+    if ((st = fused_step(m, f, FusedInput{Xs, nullptr, 0, 0, 0}, q, tp, m->t, update, nullptr, false)) !=
+        GRIDFF_OK) return st;
   } else {
     input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->Xs, rows, n_in, Mp, m->pads[0], m->H[0], m->HT[0]);
     if ((st = enqueue_train(m, n_targets, K, tors_mask != nullptr, tp, flags)) != GRIDFF_OK) return st;
@@ -1055,7 +1073,7 @@ gridff_status gridff_mlp_train(gridff_mlp* m, int32_t steps, int32_t n_targets, 
     for (int k = 0; k < steps; ++k) {
       q.base = (unsigned long long)(m->rng_step + k) << 20;
       const FusedInput in{nullptr, m->desc, n_desc, (unsigned long long)seed, q.base};
-      if ((st = fused_step(m, f, in, q, tp, m->t + k + 1, 1, m->loss_hist + k)) != GRIDFF_OK) return st;
+      if ((st = fused_step(m, f, in, q, tp, m->t + k + 1, 1, m->loss_hist + k, k > 0)) != GRIDFF_OK) return st;
     }
     m->rng_step += steps;
     m->t += steps;
@@ -1127,7 +1145,7 @@ gridff_status gridff_mlp_propose(gridff_mlp* m, gridff_replicas* R, const float*
   const int Mp = pad16(rows);
   GRIDFF_CUDA(ctx, cudaMemcpyAsync(m->desc, descriptor, n_desc * sizeof(float), cudaMemcpyHostToDevice, s));
   const float* Y = m->fused ? f.Y : m->Y;
-  if (m->fused) fused_forward(m, f, FusedInput{nullptr, m->desc, n_desc, (unsigned long long)seed, 0}, 0);
+  if (m->fused) fused_forward(m, f, FusedInput{nullptr, m->desc, n_desc, (unsigned long long)seed, 0}, 0, false);
   else {
     propose_input_kernel<<<grid1((long long)Mp * m->pads[0]), 256, 0, s>>>(m->desc, n_desc, m->sizes[0] - n_desc, rows,
                                                                            (unsigned long long)seed, Mp, m->pads[0],

@@ -88,6 +88,25 @@ __device__ __forceinline__ void ldsm4_t(const void* smem, unsigned (&r)[4]) {
                : "r"((unsigned)__cvta_generic_to_shared(smem)));
 }
 
+// The four launches of a step overlap: each is started when every block of the
+// one before has called next_may_start(), and waits in previous_done() until that
+// one has ended and its writes are visible.  next_may_start() always stands
+// behind previous_done(), so what runs ahead of the wait sees the end of
+// every launch but the one before, and runs beside that one alone: the inputs
+// (written where only the gradients read), the weights of the backward pass (the
+// forward does not write them), the optimiser's state.  At 2048 rows x
+// 80-256-256-256-19 a step took 48 us, about 6 of them between the launches; now 42.
+__device__ __forceinline__ void previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Weights are written by the launch before: an ordinary load that stays behind
+// previous_done() (a read-only load may not be used while another grid writes).
+__device__ __forceinline__ uint4 load_weights(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
 // A warp's share of a product: the n8 tiles w + 8 c (c < 4, below nt) of the
 // fragment-ordered operand B, k = 0 .. 32 kp - 1.  The whole share of a layer (up
 // to 128 registers) is requested at once and one layer ahead: the weights come
@@ -98,16 +117,17 @@ struct RowsB {
 };
 // FULL: 256 inputs and 256 outputs, no tile of the share is missing.
 template <bool FULL>
-__device__ __forceinline__ void rows_load_t(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
+__device__ __forceinline__ void rows_load_t(RowsB& B, const __nv_bfloat16* W, int kp, int nt, int w, int lane) {
   const uint4* b = (const uint4*)W + lane;
 #pragma unroll
   for (int p = 0; p < kFusedW / 32; ++p)
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (FULL || (p < kp && w + 8 * c < nt)) B.v[c][p] = __ldg(b + ((w + 8 * c) * (FULL ? kFusedW / 32 : kp) + p) * 32);
+      if (FULL || (p < kp && w + 8 * c < nt)) 
+        B.v[c][p] = load_weights(b + ((w + 8 * c) * (FULL ? kFusedW / 32 : kp) + p) * 32);
 }
 __device__ __forceinline__ bool rows_full(int kp, int nt) { return kp == kFusedW / 32 && nt == kFusedW / 8; }
-__device__ __forceinline__ void rows_load(RowsB& B, const __nv_bfloat16* __restrict__ W, int kp, int nt, int w, int lane) {
+__device__ __forceinline__ void rows_load(RowsB& B, const __nv_bfloat16* W, int kp, int nt, int w, int lane) {
   if (rows_full(kp, nt)) rows_load_t<true>(B, W, kp, nt, w, lane);
   else rows_load_t<false>(B, W, kp, nt, w, lane);
 }
@@ -153,8 +173,7 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
                                       (__nv_bfloat16 (*)[kFusedLd])(smem_h + (size_t)16 * MT * kFusedLd)};
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int m0 = blockIdx.x * 16 * MT;
-  RowsB B;
-  rows_load(B, net.Wf[0], k32(net.pad[0]), net.pad[1] >> 3, w, lane);
+  if (in.X) previous_done();          // rows from memory: the launch before may write them
   {
     const int ip = net.pad[0], ip32 = 32 * k32(ip), n_in = net.size[0];
     // 16 threads a row, columns 16 apart: the noise inputs (a logarithm, a square
@@ -173,6 +192,10 @@ __global__ void __launch_bounds__(256) fused_forward_kernel(FusedNet net, FusedI
         if (train && k < ip && m < net.Mp) net.H[0][(size_t)m * ip + k] = b;
       }
   }
+  previous_done();
+  next_may_start();
+  RowsB B;
+  rows_load(B, net.Wf[0], k32(net.pad[0]), net.pad[1] >> 3, w, lane);
   __syncthreads();
   for (int l = 0; l < net.L; ++l) {
     const int op = net.pad[l + 1], nt = op >> 3, n_out = net.size[l + 1], cur = l & 1;
@@ -254,6 +277,8 @@ __global__ void __launch_bounds__(256) fused_backward_kernel(FusedNet net, Fused
   if (L > 1) rows_load(B, net.Wr[L - 1], k32(opl), net.pad[L - 1] >> 3, w, lane);
   if (tid < nb) s_row[tid] = target_row(q, ba + tid);
   for (int e = tid; e < 16 * 32 * k32(opl); e += 256) sG[0][e / (32 * k32(opl))][e % (32 * k32(opl))] = __float2bfloat16(0.f);
+  previous_done();
+  next_may_start();
   __syncthreads();
   const float* Yb = net.Y + (size_t)ba * K * n_out;
   if (q.mask)
@@ -378,6 +403,8 @@ constexpr int kGLd = 72;          // 64 columns + 8: rows 144 B apart, conflict-
 __global__ void __launch_bounds__(128) fused_grad_kernel(FusedNet net, GradMap map) {
   __shared__ __align__(16) __nv_bfloat16 sA[2][32][kGLd], sB[2][32][kGLd];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  previous_done();
+  next_may_start();
   if ((int)blockIdx.x >= map.first[net.L]) {
     // part[chunk][j] = sum over the chunk's rows of G[m][j]
     int l = 0;
@@ -486,9 +513,10 @@ struct AdamArgs {
 // Gradient of every parameter (parts added in order), Adam, the operands, and
 // (last block) the mean loss of the step.
 __global__ void __launch_bounds__(256) fused_update_kernel(FusedNet net, AdamArgs ad, int n_params,
-                                                           const float* __restrict__ loss, int n_targets,
-                                                           float* __restrict__ hist) {
+                                                           const float* loss, int n_targets, float* hist) {
   if (blockIdx.x == gridDim.x - 1) {
+    previous_done();
+    next_may_start();
     if (!hist) return;
     __shared__ float part[256];
     float s = 0.f;
@@ -503,6 +531,14 @@ __global__ void __launch_bounds__(256) fused_update_kernel(FusedNet net, AdamArg
     return;
   }
   const int p = blockIdx.x * 256 + threadIdx.x;
+  float m0 = 0.f, v0 = 0.f, x0 = 0.f;
+  if (p < n_params && ad.update) {
+    m0 = net.Am[p];
+    v0 = net.Av[p];
+    x0 = net.P[p];
+  }
+  previous_done();
+  next_may_start();
   if (p >= n_params) return;
   int l = 0;
   while (l + 1 < net.L && (size_t)p >= net.woff[l + 1]) ++l;
@@ -524,11 +560,12 @@ __global__ void __launch_bounds__(256) fused_update_kernel(FusedNet net, AdamArg
   }
   net.Gr[p] = g;
   if (!ad.update) return;
-  const float m = ad.b1 * net.Am[p] + (1.f - ad.b1) * g;
-  const float v = ad.b2 * net.Av[p] + (1.f - ad.b2) * g * g;
+  // the contractions written out: the bits of adam_kernel
+  const float m = fmaf(1.f - ad.b1, g, ad.b1 * m0);
+  const float v = fmaf((1.f - ad.b2) * g, g, ad.b2 * v0);
   net.Am[p] = m;
   net.Av[p] = v;
-  const float x = net.P[p] - ad.c1 * m / (sqrtf(v * ad.c2) + ad.eps);
+  const float x = x0 - ad.c1 * m / (sqrtf(v * ad.c2) + ad.eps);
   net.P[p] = x;
   if (!bias) put_weight(net, l, o, i, x);
 }
