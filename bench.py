@@ -225,23 +225,22 @@ def run_reference(args):
 def kernel_source_hash():
     """Hash of the source the rigid sub-warp relaxation kernel is built
     from: the shared headers (internal.h, interp.cuh: cell location and
-    B-spline weights), the device helpers at the top of dynamics.cu (record
-    gathers), the final-evaluation record and the sub-warp section (force
-    routine, schedule, kernel).  Edits elsewhere in the file (flexible
-    kernels, host code) leave the committed counters valid."""
+    B-spline weights, replica_common.cuh: record gathers), and of dynamics.cu
+    the final-evaluation record and the sub-warp section (force routine,
+    schedule, kernel).  Edits elsewhere in the file (flexible kernels, host
+    code) leave the committed counters valid."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2508_15522_gb300", "csrc")
-    for name in ("internal.h", "interp.cuh"):
+    for name in ("internal.h", "interp.cuh", "replica_common.cuh"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
     src = open(os.path.join(csrc, "dynamics.cu"), encoding="utf-8").read()
     try:
-        top = src[:src.index("// Energy and force of one atom in the substrate field")]
         r0 = src.index("// Record of a replica's final evaluation")
         r1 = src.index("// Forces of one flexible replica whose positions are in s.x", r0)
         a = src.index("// FIRE, rigid replicas, sub-warp form")
         b = src.index("// FIRE, flexible replicas", a)
-        h.update((top + src[r0:r1] + src[a:b]).encode())
+        h.update((src[r0:r1] + src[a:b]).encode())
     except ValueError:
         h.update(src.encode())
     return h.hexdigest()[:16]

@@ -1084,10 +1084,11 @@ gridff_status gridff_mlp_train(gridff_mlp* m, int32_t steps, int32_t n_targets, 
   }
   if (!m->ctr && dalloc(m, &m->ctr, 1) != cudaSuccess) return set_err(ctx, GRIDFF_ENOMEM, "step counters");
   if (m->fused) refresh_layers(m);
-  // The loop is launch-bound (about 45 small launches per step), so one step
-  // is captured in a CUDA graph and replayed `steps` times; everything that
-  // changes between steps (random-stream step, history slot, Adam t and its
-  // factors) lives in device counters advanced by the graph's first node.
+  // Networks that the fused step does not take: about 45 small launches per
+  // step, bound by their launches, so one step is captured in a CUDA graph and
+  // replayed `steps` times; everything that changes between steps (random-stream
+  // step, history slot, Adam t and its factors) lives in device counters advanced
+  // by the graph's first node.
   StepCounters c0{};
   c0.next_step = m->rng_step;
   c0.t = m->t;
