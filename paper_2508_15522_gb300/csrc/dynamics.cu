@@ -287,12 +287,15 @@ __device__ __forceinline__ Acc flex_forces(const GridView& g, bool use_grid, boo
 // (Morse with mixed R_i + R_j and eps_i eps_j, plus Coulomb), from per-atom
 // factors prepared once per replica: pi = {k_e q_i, a R_i, eps_i, -} for
 // this lane's atom and pj = {q_j, a R_j, eps_j, -} for the partner, with
-// a = alpha log2(e), so that e^{-alpha (r - R_i - R_j)} = 2^{a R_i + a R_j - a r}.
+// a = alpha log2(e), so that e^{-alpha (r - R_i - R_j)} = 2^{a R_i + a R_j - a r};
+// EX (evaluations and constant-energy dynamics, whose energies are summed in
+// FP64): R_i and R_j as they are and expf (pair_exp()).
+template <bool EX>
 __device__ __forceinline__ void nb_pair(float3 d, float4 pi, float4 pj, float alpha, float a, float& c, float& e) {
   const float r2 = dot3(d, d);
   const float ir = rsqrtf(r2);
   const float r = r2 * ir;
-  const float e1 = ex2_approx(fmaf(-a, r, pi.y + pj.y));
+  const float e1 = pair_exp<EX>(alpha, a, r, pi.y, pj.y);
   const float ee = pi.z * pj.z;
   const float qr = pi.x * pj.x * ir;                      // k_e q_i q_j / r
   c = -(2.f * alpha * ee * e1 * (1.f - e1) - qr * ir) * ir;
@@ -320,7 +323,7 @@ __device__ __forceinline__ void pad_pair_slots(float* s_x, float4* s_nb, int n, 
 // bit d of act is set.  Slots from n to the next multiple of 32 hold zero
 // positions and factors (written when the replica is loaded).  Adds the pair forces to fi and the energies to e;
 // returns the reactions received on this lane's atom of the partner block.
-template <bool DIAG>
+template <bool DIAG, bool EX>
 __device__ __forceinline__ float3 nb_steps(const float* s_x, const float4* s_nb, float3 xi, float4 pi, float alpha,
                                            float a, uint32_t act, int lane, int base, int ring, int d0, int d1,
                                            float3& fi, float& e) {
@@ -334,7 +337,7 @@ __device__ __forceinline__ float3 nb_steps(const float* s_x, const float4* s_nb,
     const int j = base + sl;
     const float3 dv = sub3(xi, ld3(s_x, j));
     float c, ep;
-    nb_pair(dv, pi, s_nb[j], alpha, a, c, ep);
+    nb_pair<EX>(dv, pi, s_nb[j], alpha, a, c, ep);
     c = on ? c : 0.f;                      // slots past n hold zeros: dv stays finite
     const float cx = c * dv.x, cy = c * dv.y, cz = c * dv.z;
     e += on ? ep : 0.f;
@@ -398,12 +401,12 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
         const int h = m >> 1;
         act &= ((2u << h) - 1u) & ~1u;                          // d = 1 .. m/2
         if (!(m & 1) && lane >= h) act &= ~(1u << h);           // d = m/2 counted from l < m/2
-        gj = nb_steps<true>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, ring, 1, h, fi, e);
+        gj = nb_steps<true, kExactExp<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, ring, 1, h, fi, e);
         fi.x += gj.x;
         fi.y += gj.y;
         fi.z += gj.z;
       } else {
-        gj = nb_steps<false>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, 32, 0, 31, fi, e);
+        gj = nb_steps<false, kExactExp<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, 32, 0, 31, fi, e);
         if (base + lane < n) {
           float* f = s_f + 3 * (base + lane);
           f[0] += gj.x;
@@ -600,11 +603,7 @@ eval_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
       }
     } else {
       for (int m = lane; m < 3 * n; m += 32) s.x[m] = xs[3 * (size_t)off + m];
-      for (int i = lane; i < n; i += 32) {
-        float4 p = __ldg(&tv.nb[ab + i]);
-        p.y *= tv.alpha * kLog2e;
-        s_nb[i] = p;
-      }
+      for (int i = lane; i < n; i += 32) s_nb[i] = __ldg(&tv.nb[ab + i]);
       pad_pair_slots(s.x, s_nb, n, lane);
     }
     int flags = 0;
@@ -1606,11 +1605,11 @@ md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
       s.x[m] = xs[3 * (size_t)off + m];
       s.v[m] = vs[3 * (size_t)off + m];
     }
-    // nonbonded factors {q, alpha log2(e) R, eps} and 1/m or 1/sqrt(m) in the
+    // nonbonded factors {q, alpha log2(e) R (NVE: R), eps} and 1/m or 1/sqrt(m) in the
     // free fourth slot; zeros up to the next multiple of 32 atoms
     for (int i = lane; i < n; i += 32) {
       float4 p = __ldg(&tv.nb[ab + i]);
-      p.y *= tv.alpha * kLog2e;
+      if (!NVE) p.y *= tv.alpha * kLog2e;
       const float mass = __ldg(&tv.body[ab + i]).w;
       p.w = NVE ? 1.f / mass : rsqrtf(mass);
       s_nb[i] = p;

@@ -56,7 +56,7 @@ struct TeamArgs {
 struct TeamState {
   StencilCache sc;
   float4* x;        // [N] {x, y, z, q}
-  float2* nb;       // [N] {alpha log2(e) R, eps}
+  float2* nb;       // [N] {alpha log2(e) R, eps} (TEAM_NVE, TEAM_EVAL: {R, eps})
   float* im;        // [N] 1/m, or 1/sqrt(m) (Langevin)
   float* v;         // [3N]
   float* f;         // [3N] grid force, then the total
@@ -178,7 +178,7 @@ __device__ __forceinline__ Acc team_pairs(const TeamState& s, const TemplateView
         const float3 dv = sub3(xi, xyz(P));
         const float r2 = dot3(dv, dv);
         const float ir = rsqrtf(r2), r = r2 * ir;
-        const float e1 = ex2_approx(fmaf(-a, r, p2.x + Q.x));
+        const float e1 = pair_exp<kExactExp<Acc>>(alpha, a, r, p2.x, Q.x);
         const float ee = p2.y * Q.y, qr = qi * P.w * ir;      // k_e q_i q_j / r
         const bool on = act & 1u;
         act >>= 1;
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
       const float m = in ? __ldg(&tv.body[ab + i]).w : 1.f;
       const float* x = A.xs + 3 * ((size_t)off + i);
       s.x[i] = in ? make_float4(x[0], x[1], x[2], p.x) : p;
-      s.nb[i] = make_float2(p.y * (tv.alpha * kLog2e), p.z);
+      s.nb[i] = make_float2(kExactExp<Acc> ? p.y : p.y * (tv.alpha * kLog2e), p.z);
       s.im[i] = MODE == TEAM_LANGEVIN ? rsqrtf(m) : 1.f / m;
       for (int c = 0; c < 3; ++c) s.v[3 * i + c] = in && MODE != TEAM_EVAL ? A.vs[3 * ((size_t)off + i) + c] : 0.f;
     }
