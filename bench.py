@@ -231,9 +231,11 @@ def kernel_source_hash():
     code) leave the committed counters valid."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2508_15522_gb300", "csrc")
-    for name in ("internal.h", "interp.cuh", "replica_common.cuh"):
+    for name in ("internal.h", "interp.cuh"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
+    common = open(os.path.join(csrc, "replica_common.cuh"), encoding="utf-8").read()
+    h.update(common.split("// 2^x by the PTX instruction")[0].encode())   # before the pair exponential
     src = open(os.path.join(csrc, "dynamics.cu"), encoding="utf-8").read()
     try:
         r0 = src.index("// Record of a replica's final evaluation")
