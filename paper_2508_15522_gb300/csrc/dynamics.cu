@@ -401,12 +401,12 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
         const int h = m >> 1;
         act &= ((2u << h) - 1u) & ~1u;                          // d = 1 .. m/2
         if (!(m & 1) && lane >= h) act &= ~(1u << h);           // d = m/2 counted from l < m/2
-        gj = nb_steps<true, kExactExp<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, ring, 1, h, fi, e);
+        gj = nb_steps<true, kReadOut<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, ring, 1, h, fi, e);
         fi.x += gj.x;
         fi.y += gj.y;
         fi.z += gj.z;
       } else {
-        gj = nb_steps<false, kExactExp<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, 32, 0, 31, fi, e);
+        gj = nb_steps<false, kReadOut<Acc>>(s_x, s_nb, xi, pi, alpha, a2, act, lane, base, 32, 0, 31, fi, e);
         if (base + lane < n) {
           float* f = s_f + 3 * (base + lane);
           f[0] += gj.x;
@@ -428,14 +428,13 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   __syncwarp();
   // Bonded terms (few per atom): lanes take terms round-robin and add the
   // forces with shared-memory atomics.  Reciprocals come from rsqrtf
-  // (1/x = rsqrt(x)^2), not from divisions.
+  // (1/x = rsqrt(x)^2), not from divisions, except where results are read
+  // (bond_factor()).
   for (int b = tv.ub_off[t] + lane; b < tv.ub_off[t + 1]; b += 32) {
     const BondTerm B = tv.ub[b];
     const float3 d = sub3(ld3(s_x, B.i), ld3(s_x, B.j));
-    const float r2 = dot3(d, d);
-    const float ir = r2 > 0.f ? rsqrtf(r2) : 0.f;   // zero length: no direction, no force
-    const float dr = r2 * ir - B.r0;
-    const float c = -2.f * B.k * dr * ir;
+    float c, dr;
+    bond_factor<kReadOut<Acc>>(dot3(d, d), B.k, B.r0, c, dr);
     sh_add3(s_f, B.i, c * d.x, c * d.y, c * d.z);
     sh_add3(s_f, B.j, -c * d.x, -c * d.y, -c * d.z);
     e += B.k * dr * dr;
@@ -443,8 +442,8 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   for (int a = tv.ua_off[t] + lane; a < tv.ua_off[t + 1]; a += 32) {
     const AngleRec A = tv.ua[a];
     const float3 u = sub3(ld3(s_x, A.a), ld3(s_x, A.b)), w = sub3(ld3(s_x, A.c), ld3(s_x, A.b));
-    const float ru = rsqrtf(dot3(u, u)), rw = rsqrtf(dot3(w, w));
-    const float inv = ru * rw, iu2 = ru * ru, iw2 = rw * rw;
+    const float u2 = dot3(u, u), w2 = dot3(w, w), ru = rsqrtf(u2), rw = rsqrtf(w2);
+    const float inv = kReadOut<Acc> ? rsqrtf(u2 * w2) : ru * rw, iu2 = ru * ru, iw2 = rw * rw;
     const float c = dot3(u, w) * inv;
     const float dEdc = 2.f * A.k * (c - A.cos0);
     const float cu = c * iu2, cw = c * iw2;

@@ -178,7 +178,7 @@ __device__ __forceinline__ Acc team_pairs(const TeamState& s, const TemplateView
         const float3 dv = sub3(xi, xyz(P));
         const float r2 = dot3(dv, dv);
         const float ir = rsqrtf(r2), r = r2 * ir;
-        const float e1 = pair_exp<kExactExp<Acc>>(alpha, a, r, p2.x, Q.x);
+        const float e1 = pair_exp<kReadOut<Acc>>(alpha, a, r, p2.x, Q.x);
         const float ee = p2.y * Q.y, qr = qi * P.w * ir;      // k_e q_i q_j / r
         const bool on = act & 1u;
         act >>= 1;
@@ -209,6 +209,7 @@ __device__ __forceinline__ Acc team_pairs(const TeamState& s, const TemplateView
 // Bonded terms of template t, one per thread of the team: forces on the term's
 // atoms to the term's slots (bonds: the force on atom i; angles: a, b, c;
 // torsions: a, b, c, d).  Returns this thread's share of the energy.
+template <bool EX>
 __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateView& tv, int t, int tid, int threads) {
   const int b0 = tv.ub_off[t], a0 = tv.ua_off[t], k0 = tv.ut_off[t];
   const int nb = tv.ub_off[t + 1] - b0, na = tv.ua_off[t + 1] - a0, nt = tv.ut_off[t + 1] - k0;
@@ -249,8 +250,8 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
       const AngleRec A = tv.ua[a0 + j];
       const float3 xb = xyz(s.x[A.b]);
       const float3 u = sub3(xyz(s.x[A.a]), xb), w = sub3(xyz(s.x[A.c]), xb);
-      const float ru = rsqrtf(dot3(u, u)), rw = rsqrtf(dot3(w, w));
-      const float inv = ru * rw, iu2 = ru * ru, iw2 = rw * rw;
+      const float u2 = dot3(u, u), w2 = dot3(w, w), ru = rsqrtf(u2), rw = rsqrtf(w2);
+      const float inv = EX ? rsqrtf(u2 * w2) : ru * rw, iu2 = ru * ru, iw2 = rw * rw;
       const float c = dot3(u, w) * inv;
       const float dEdc = 2.f * A.k * (c - A.cos0);
       const float cu = c * iu2, cw = c * iw2;
@@ -264,10 +265,8 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
       const int j = k - nt - na;
       const BondTerm B = tv.ub[b0 + j];
       const float3 d = sub3(xyz(s.x[B.i]), xyz(s.x[B.j]));
-      const float r2 = dot3(d, d);
-      const float ir = r2 > 0.f ? rsqrtf(r2) : 0.f;   // zero length: no direction, no force
-      const float dr = r2 * ir - B.r0;
-      const float c = -2.f * B.k * dr * ir;
+      float c, dr;
+      bond_factor<EX>(dot3(d, d), B.k, B.r0, c, dr);
       put3(s.slot, j, c * d.x, c * d.y, c * d.z);
       e += B.k * dr * dr;
     }
@@ -305,7 +304,7 @@ __device__ __forceinline__ Acc team_forces(const GridView& g, const TemplateView
   float* const fw = s.fw + (size_t)w * 3 * A.N;
   if (A.use_intra) {
     e += team_pairs<NW, Acc>(s, tv, ab, n, lane, w, fw);
-    e += (Acc)team_bonded(s, tv, t, tid, 32 * NW);
+    e += (Acc)team_bonded<kReadOut<Acc>>(s, tv, t, tid, 32 * NW);
   }
   __syncthreads();
   f2 = P = v2 = 0.f;
@@ -425,7 +424,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
       const float m = in ? __ldg(&tv.body[ab + i]).w : 1.f;
       const float* x = A.xs + 3 * ((size_t)off + i);
       s.x[i] = in ? make_float4(x[0], x[1], x[2], p.x) : p;
-      s.nb[i] = make_float2(kExactExp<Acc> ? p.y : p.y * (tv.alpha * kLog2e), p.z);
+      s.nb[i] = make_float2(kReadOut<Acc> ? p.y : p.y * (tv.alpha * kLog2e), p.z);
       s.im[i] = MODE == TEAM_LANGEVIN ? rsqrtf(m) : 1.f / m;
       for (int c = 0; c < 3; ++c) s.v[3 * i + c] = in && MODE != TEAM_EVAL ? A.vs[3 * ((size_t)off + i) + c] : 0.f;
     }
