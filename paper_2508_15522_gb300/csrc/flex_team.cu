@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
   for (int j = blockIdx.x;; j += gridDim.x) {
     int k = j;
     if (queued) {
-      if (tid == 0) *s.word = atomicAdd(&ctl.res->next, 1);
+      if (tid == 0) *s.word = atomicAdd(&ctl.res->team_next, 1);
       __syncthreads();
       k = *s.word;
       __syncthreads();

@@ -168,7 +168,7 @@ struct DevResult {
   int max_steps;
   int next;           // work-queue position (replicas handed out so far)
   int handoff_timeouts;   // split relaxations whose first part did not arrive in time
-  int pad;
+  int team_next;      // the same of the team kernel: both run in a call whose batch is split
 };
 
 // Launch configuration of a relaxation (mirrors gridff_launch_config).
