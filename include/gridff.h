@@ -63,9 +63,9 @@ typedef enum {
   GRIDFF_EABORTED = 4,    /* the host abort flag stopped a relax/run call */
   GRIDFF_ESTEPLIMIT = 5,  /* the clock budget of a relax/run call ran out */
   GRIDFF_ENOTSUP = 6,     /* combination the library does not support */
-  GRIDFF_ETIMEOUT = 7     /* a bounded wait inside a kernel ran out (a relaxation split across
-                             two warps did not receive its first part in time); the replicas
-                             concerned keep the state of that first part */
+  GRIDFF_ETIMEOUT = 7     /* a bounded wait inside a kernel ran out (a relaxation cut into parts
+                             for several warps saw no part end for a second); the replicas
+                             concerned keep the state of the last part that ended */
 } gridff_status;
 
 /* per-replica status bits (status_out arrays, gridff_get_fire_state).  A
@@ -88,8 +88,8 @@ typedef enum {
 #define GRIDFF_NO_INTRA 16       /* eval/relax/run: skip the intramolecular terms */
 #define GRIDFF_POINTS_BINNED 32  /* eval_points: put the points in cell order on the device first */
 #define GRIDFF_TEST_NO_HANDOFF 256  /* relax (rigid sub-warp layout), test hook of the bounded wait:
-                                       the first parts of split relaxations publish no hand-off,
-                                       so their second parts give up after about a second and the
+                                       the parts of split relaxations publish no hand-off, so
+                                       their later parts give up after about a second and the
                                        call returns GRIDFF_ETIMEOUT; the context stays usable */
 
 /* grid channels */
@@ -410,9 +410,9 @@ gridff_status gridff_template_factors(const gridff_replicas* reps, int32_t t, fl
  * does not depend on the layout or schedule beyond FP32 summation order
  * (rigid layouts: bit for bit).
  * Errors: EINVAL, ECUDA, EABORTED, ESTEPLIMIT (state is consistent),
- * ETIMEOUT (rigid sub-warp layout: a split relaxation's second part gave up
- * waiting for its first; the replicas concerned keep the first part's
- * state). */
+ * ETIMEOUT (rigid sub-warp layout: a later part of a relaxation cut into parts
+ * gave up waiting for the parts before it; the replicas concerned keep the state of
+ * the last part that ended). */
 gridff_status gridff_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* reps,
                            int32_t nsteps, const gridff_fire_params* params, int flags,
                            gridff_relax_result* result);
@@ -441,7 +441,8 @@ typedef struct {
                                  steps); 0 = no staging, every gather from L2/HBM */
   int32_t queue;              /* FLEX_TERMS: 1 = replicas handed out by an atomic work queue in
                                  decreasing cost order (uneven sizes), 0 = static round robin.
-                                 RIGID_SUBWARP: 1 = warp tasks handed out by an atomic queue,
+                                 RIGID_SUBWARP: 1 = warp tasks handed out by an atomic queue (in
+                                 parts of equal iteration ranges when they outnumber the warps),
                                  2 = the (task, iteration) grid cut into equal ranges per warp (a
                                  task may be split between two warps), 0 = per call: the queue
                                  when f_conv > 0 (replicas may stop early), else the ranges */

@@ -1019,12 +1019,16 @@ __device__ __noinline__ SwPart sw_part(int warp, int n_warps, int P, int nsteps,
   return s;
 }
 
-// Bound of the wait for a hand-off flag: one second of %globaltimer time,
-// after which the part is skipped and the call returns GRIDFF_ETIMEOUT.
-// The poll count is only a backstop that ends the loop should the timer
-// not advance (polls are about a microsecond apart: an acquire load from
-// L2 and a requested 1 us sleep).  A head finishes a quarter of a task
-// before its tail starts, so a working launch never waits long.
+// Bound of the wait for a hand-off flag: one second of %globaltimer time per
+// part, after which the waiting part is skipped and the call returns
+// GRIDFF_ETIMEOUT.  The flag counts the task's ended parts, and a later part
+// waits for all before it, so the second begins anew whenever the count rises:
+// when most tasks have converged, idle warps hold every remaining part of a slow
+// one, and the last of them waits for almost the whole relaxation.  The poll
+// count is only a backstop that ends the loop should the timer not advance (polls are
+// about a microsecond apart: an acquire load from L2 and a requested 1 us
+// sleep).  A head of the time-sliced ranges finishes a quarter of a task before
+// its tail starts, so a working launch never waits long there.
 constexpr unsigned long long kHandoffWaitNs = 1000000000ull;
 constexpr int kHandoffPolls = 1 << 23;
 
@@ -1038,13 +1042,22 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 }
 
 // The hand-off flag's value once it counts `parts` ended parts (bits 0 .. 15),
-// or its last value when the bounded wait ran out (one lane calls it).
+// or its last value when the bounded wait ran out (one lane calls it).  The
+// count rises at most `parts` times: the loop ends.
 __device__ __noinline__ int wait_handoff(const int* flag, int parts) {
-  const unsigned long long deadline = gtimer() + kHandoffWaitNs;
-  int hv = 0;
+  unsigned long long deadline = gtimer() + kHandoffWaitNs;
+  int hv = 0, seen = 0;
   for (int k = 0; k < kHandoffPolls; ++k) {
     hv = ld_acquire(flag);
-    if ((hv & 0xffff) >= parts || gtimer() > deadline) break;
+    const int ended = hv & 0xffff;
+    if (ended >= parts) break;
+    const unsigned long long now = gtimer();
+    if (ended > seen) {
+      seen = ended;
+      deadline = now + kHandoffWaitNs;
+      k = 0;
+    }
+    if (now > deadline) break;
     __nanosleep(1000);
   }
   return hv;
@@ -2420,7 +2433,8 @@ cudaError_t launch_ex(void (*fn)(KArgs...), int blocks, int threads, size_t dyn,
 // 1.68 of work); with C parts per task the rounds are ceil(C tasks / warps) / C.
 // A part costs about one and a half iterations more (its state through L2, every
 // stencil of its atoms refilled), so C minimises the sum.  Parts are at most 4096
-// iterations (0.2 s of the largest molecules), well inside the bounded wait.
+// iterations (0.2 s of the largest molecules): the bounded wait counts anew with
+// every part that ends.
 // 4096 x 38 atoms, 200 iterations a call: 1189 -> 1073 us (4 parts).
 static int sw_queue_parts(long long tasks, long long warps, int nsteps) {
   if (tasks <= warps) return 1;
