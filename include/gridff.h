@@ -501,7 +501,7 @@ gridff_status gridff_relax_graph_create(gridff_ctx* ctx, const gridff_grid* grid
                                         int32_t nsteps, const gridff_fire_params* params, int flags,
                                         gridff_graph** out);
 /* Replay.  result != NULL: wait for it and fill result (as gridff_relax,
- * including EABORTED/ESTEPLIMIT); result == NULL: return after enqueueing. */
+ * including EABORTED/ESTEPLIMIT/ETIMEOUT); result == NULL: return after enqueueing. */
 gridff_status gridff_graph_launch(gridff_graph* graph, gridff_relax_result* result);
 void gridff_graph_destroy(gridff_graph* graph);
 

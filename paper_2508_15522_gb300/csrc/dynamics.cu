@@ -2257,7 +2257,7 @@ gridff_status finish_launch(gridff_ctx* ctx, DevResult* hres) {
   if (hres->stop_bits & GRIDFF_REP_STEPLIMIT)
     return set_err(ctx, GRIDFF_ESTEPLIMIT, "clock budget exhausted");
   if (hres->handoff_timeouts)
-    return set_err(ctx, GRIDFF_ETIMEOUT, "%d split relaxations did not receive their first part in time",
+    return set_err(ctx, GRIDFF_ETIMEOUT, "%d parts of split relaxations did not receive the one before in time",
                    hres->handoff_timeouts);
   return GRIDFF_OK;
 }

@@ -339,6 +339,9 @@ gridff_status gridff_graph_launch(gridff_graph* G, gridff_relax_result* result) 
   result->max_steps = h.max_steps;
   if (h.stop_bits & GRIDFF_REP_ABORTED) return set_err(ctx, GRIDFF_EABORTED, "aborted by the host flag");
   if (h.stop_bits & GRIDFF_REP_STEPLIMIT) return set_err(ctx, GRIDFF_ESTEPLIMIT, "clock budget exhausted");
+  if (h.handoff_timeouts)
+    return set_err(ctx, GRIDFF_ETIMEOUT, "%d parts of split relaxations did not receive the one before in time",
+                   h.handoff_timeouts);
   return GRIDFF_OK;
 }
 

@@ -1,5 +1,5 @@
 """The bounded wait of the rigid queue's hand-off bounds one part, not all parts
-before it."""
+before it, and a captured relaxation reports a wait that ran out."""
 import numpy as np
 import pytest
 
@@ -43,3 +43,22 @@ def test_a_straggler_may_take_longer_than_the_wait(env):
     assert st == G.OK and steps[0] == nsteps and (steps[1:] == 1).all()
     assert ctx.last_kernel_ms() > 1200.0          # else the case does not reach the wait
     assert res.n_converged == n_rep - 1
+
+
+def test_a_captured_relaxation_reports_the_wait(env):
+    """With the hook that publishes no hand-off, the second parts give up (6 tasks cut
+    into ranges for 4 warps); the replay says so as the direct call does."""
+    G, ctx, sub, grid, sms = env
+    mol = synth.c24h8o6_core()
+    com, quat = synth.rigid_poses(mol, sub, 11, seed=2)
+    reps = G.Replicas(ctx, [mol], [0] * 11, rigid=True)
+    cfg = reps.launch_config()
+    cfg.lanes_per_replica, cfg.blocks, cfg.queue = 16, 1, 2
+    reps.set_launch_config(cfg)
+    reps.set_state(np.concatenate([com, quat], 1).astype(np.float32).ravel())
+    graph = G.RelaxGraph(ctx, grid, reps, 100, G.fire_params(f_conv=0.0), flags=G.TEST_NO_HANDOFF)
+    st, _ = graph.launch(check=False)
+    assert st == G.ETIMEOUT
+    graph.close()
+    st, res = G.relax(ctx, grid, reps, 100, G.fire_params(f_conv=0.0), check=False)
+    assert st == G.OK and res.atom_evals == 11 * mol.n * 100
