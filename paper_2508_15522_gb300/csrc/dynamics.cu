@@ -1447,7 +1447,7 @@ relax_flex_terms_kernel(GridView g, TemplateView tv, const int* __restrict__ rep
   float4* s_nb = (float4*)(wbase + cache_bytes(S));
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
-  const unsigned long long t0 = gtimer();
+  const unsigned long long t0 = lane == 0 ? budget_start(ctl) : 0;
   for (int k = warp;; k += n_warps) {
     if (order) {
       int next = 0;
@@ -1593,7 +1593,7 @@ md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
   float4* s_nb = (float4*)(wbase + cache_bytes(S));
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
-  const unsigned long long t0 = gtimer();
+  const unsigned long long t0 = lane == 0 ? budget_start(ctl) : 0;
   const float hdt = 0.5f * dt;
   const float sq_kT = sqrtf(kT_acc);
   for (int k = warp;; k += n_warps) {

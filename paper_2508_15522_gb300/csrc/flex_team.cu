@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
   constexpr int kThr = 32 * NW;
   const int tid = threadIdx.x;
   TeamState s = team_state(dyn_smem, NW, A.N, A.S, A.n_slots);
-  const unsigned long long t0 = gtimer();
+  const unsigned long long t0 = MODE != TEAM_EVAL && tid == 0 ? budget_start(ctl) : 0;
   // stop bits every 32 steps (abort flag, clock budget), the same in every thread
   auto stop = [&]() {
     if (tid == 0) {

@@ -34,6 +34,15 @@ __device__ __forceinline__ unsigned long long gtimer() {
   return t;
 }
 
+// Start of the clock budget: the same for both kernels of a split flexible
+// call, which run one after the other (the first thread here sets it).
+__device__ __forceinline__ unsigned long long budget_start(const Control& ctl) {
+  const unsigned long long t = gtimer();
+  if (!ctl.budget_ns) return t;
+  const unsigned long long first = atomicCAS(&ctl.res->t0, 0ull, t);
+  return first ? first : t;
+}
+
 __device__ __forceinline__ float wsum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);

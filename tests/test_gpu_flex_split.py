@@ -2,7 +2,7 @@
 cost order go to the warp kernel, the others to teams, within one call.  With
 molecules whose teams do not all fit the chip at once, every replica is still
 served exactly once, by relaxation, its captured graph, Langevin and NVE
-dynamics."""
+dynamics; and the two kernels share one clock budget."""
 import numpy as np
 import pytest
 
@@ -78,3 +78,27 @@ def test_every_replica_is_served_once(env, batch, call):
     assert (np.abs(e1 - e0) <= 1e-5 * np.maximum(mol.n, np.abs(e0))).all()
     if t0 is not None:
         assert (np.abs(t1 - t0) <= 1e-5 * np.maximum(mol.n, np.abs(t0))).all()
+
+
+@pytest.mark.parametrize("call", ["relax", "langevin", "run"])
+def test_one_clock_budget(env, batch, call):
+    """The budget counts from the call's first kernel: the second one, which
+    starts when the first has used it up, stops at once.  200 ms against the
+    400 ms of two budgets; 100 ms allow for the 32 steps between looks at the
+    clock (3 ms) and the launches."""
+    G, ctx, _ = env
+    mol, n_rep, x, grid = batch
+    reps = G.Replicas(ctx, [mol], [0] * n_rep)
+    for budget in (0.01, 0.2):         # the first call warms up
+        reps.set_state(x)
+        if call == "relax":
+            st, _ = G.relax(ctx, grid, reps, 10**8, G.fire_params(f_conv=0.0, clock_budget_s=budget),
+                            check=False)
+        elif call == "langevin":
+            st = G.langevin(ctx, grid, reps, 10**8, 0.1, 10.0, 0.01, seed=4, clock_budget_s=budget,
+                            check=False)
+        else:
+            st, _ = G.run(ctx, grid, reps, 10**8, 0.1, clock_budget_s=budget, check=False)
+        assert st == G.ESTEPLIMIT
+    assert 200.0 <= ctx.last_kernel_ms() <= 300.0
+    assert ((reps.fire_state()["status"] & G.REP_STEPLIMIT) != 0).all()
