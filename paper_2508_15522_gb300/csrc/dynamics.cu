@@ -2336,7 +2336,8 @@ gridff_status enqueue_md_flex(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
   const int use_grid = !(flags & GRIDFF_NO_GRID), use_intra = !(flags & GRIDFF_NO_INTRA);
   // layout: the replica set's unique-term configuration if it has one
   const LaunchCfg c = R->cfg.kernel == GRIDFF_KERNEL_FLEX_TERMS ? R->cfg : default_launch_cfg(R, true);
-  const int wpb = c.wpb, S = c.S;
+  const int wpb = c.wpb;
+  int S = c.S;
   bool gc = c.gcache && S == 0 && use_grid;
   if (gc) {
     const gridff_status gs = ensure_gcache(ctx, R);
@@ -2344,6 +2345,13 @@ gridff_status enqueue_md_flex(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
     gc = gs == GRIDFF_OK;      // NVE runs without the cache where its memory is not to be had
   }
   const MdFlexFn fn = md_flex_fn<NVE>(wpb, !grid || grid->kind == REC_F32x4, gc);
+  // a warp's velocities take shared memory that a relaxation has for stencils
+  // (5120 B of state against 3072 B): stage as many as fit, the others are gathered
+  cudaFuncAttributes fa{};
+  GRIDFF_CUDA(ctx, cudaFuncGetAttributes(&fa, (const void*)fn));
+  int optin = 0;
+  GRIDFF_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+  while (S > 0 && fa.sharedSizeBytes + flex_terms_warp_bytes(S) * wpb > (size_t)optin) --S;
   const size_t dyn = flex_terms_warp_bytes(S) * wpb;
   GRIDFF_CUDA(ctx, set_dyn_smem((const void*)fn, dyn));
   int per_sm = 0;
