@@ -2117,11 +2117,6 @@ int rigid_subwarp_width(const gridff_replicas* R) {
   return best;
 }
 
-// Allow `bytes` of dynamic shared memory (needed whenever static plus
-// dynamic shared memory exceeds 48 KB).
-cudaError_t set_dyn_smem(const void* kernel, size_t bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 int persistent_blocks(gridff_ctx* ctx, const void* kernel, int n_rep, size_t dyn_smem = 0) {
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, dyn_smem);
@@ -2353,7 +2348,7 @@ gridff_status enqueue_md_flex(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
   GRIDFF_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
   while (S > 0 && fa.sharedSizeBytes + flex_terms_warp_bytes(S) * wpb > (size_t)optin) --S;
   const size_t dyn = flex_terms_warp_bytes(S) * wpb;
-  GRIDFF_CUDA(ctx, set_dyn_smem((const void*)fn, dyn));
+  GRIDFF_CUDA(ctx, allow_dyn_smem((const void*)fn, dyn));
   int per_sm = 0;
   GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, 32 * wpb, dyn));
   if (per_sm < 1) return set_err(ctx, GRIDFF_EINVAL, "dynamics launch does not fit on an SM");
@@ -2380,7 +2375,7 @@ gridff_status prepare_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
   if (fa.sharedSizeBytes + k.dyn > (size_t)optin)
     return set_err(ctx, GRIDFF_EINVAL, "launch configuration needs %zu B of shared memory per block (limit %d)",
                    fa.sharedSizeBytes + k.dyn, optin);
-  GRIDFF_CUDA(ctx, set_dyn_smem(k.fn, k.dyn));
+  GRIDFF_CUDA(ctx, allow_dyn_smem(k.fn, k.dyn));
   int per_sm = 0;
   GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.dyn));
   if (per_sm < 1) return set_err(ctx, GRIDFF_EINVAL, "launch configuration does not fit on an SM");
@@ -2741,7 +2736,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
       // the sub-warp layout of the relaxation, every atom cached
       const int S = R->max_natoms;
       const size_t dyn = sw_warp_bytes(S, 32 / W) * kSwWarps;
-      GRIDFF_CUDA(ctx, set_dyn_smem((const void*)fn, dyn));
+      GRIDFF_CUDA(ctx, allow_dyn_smem((const void*)fn, dyn));
       const int per_block = kSwWarps * (32 / W);
       int per_sm = 0;
       GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, 32 * kSwWarps, dyn));
@@ -2762,7 +2757,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
     }
     const int S = cache_slots(R, true);
     const size_t dyn = cache_bytes(S) * kWarpsPerBlock;
-    GRIDFF_CUDA(ctx, set_dyn_smem((const void*)run_rigid_kernel, dyn));
+    GRIDFF_CUDA(ctx, allow_dyn_smem((const void*)run_rigid_kernel, dyn));
     int blocks = persistent_blocks(ctx, (const void*)run_rigid_kernel, R->n_rep, dyn);
     run_rigid_kernel<<<blocks, kThreads, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->n_rep, R->x, R->v, R->status,
                                                    R->energy, nsteps, prm->dt, rec_every, dtrace, ctl, S);

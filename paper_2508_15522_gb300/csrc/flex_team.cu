@@ -729,7 +729,7 @@ static gridff_status team_launch(gridff_ctx* ctx, const gridff_grid* grid, gridf
   A.last_f = R->last_f;
   const TeamFn fn = team_fn(NW, grid ? grid->kind : REC_F32x4, mode);
   const size_t dyn = team_bytes(NW, A.N, A.S, A.n_slots);
-  GRIDFF_CUDA(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  GRIDFF_CUDA(ctx, allow_dyn_smem((const void*)fn, dyn));
   int per_sm = 0;
   GRIDFF_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, 32 * NW, dyn));
   if (per_sm < 1) return set_err(ctx, GRIDFF_EINVAL, "team launch does not fit on an SM");

@@ -1032,7 +1032,7 @@ gridff_status gridff_build_grid(gridff_ctx* ctx, const gridff_substrate* sub,
     if (df.alloc(&d_tab, tab_bytes) != cudaSuccess) return bail(set_err(ctx, GRIDFF_ENOMEM, "radial table"));
     radial_table_kernel<<<(std::max(nt.n_f, nt.n_g) + 63) / 64, 64, 0, s>>>(nt.n_f, nt.n_g, alpha, beta, d_tab);
     nt.tab = d_tab;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tab_bytes) != cudaSuccess)
+    if (allow_dyn_smem(fn, tab_bytes) != cudaSuccess)
       return bail(set_err(ctx, GRIDFF_ECUDA, "radial table of %zu bytes", tab_bytes));
     node_values_kernel<true><<<ctx->n_sm, 32 * kNodeWarps, tab_bytes, s>>>(p, nt, d_next, vals);
   } else {

@@ -233,6 +233,23 @@ cudaError_t scratch_alloc(gridff_ctx* ctx, T** p, size_t bytes) {
   return cudaMallocFromPoolAsync((void**)p, bytes, ctx->pool, ctx->stream);
 }
 
+// Allow a launch of `kernel` with `bytes` of dynamic shared memory (needed
+// whenever static plus dynamic shared memory exceeds 48 KB).  The limit belongs to
+// the kernel, not to the launch, and calls of other threads may need more at the same
+// time: it is only ever raised, to what the device allows.
+inline cudaError_t allow_dyn_smem(const void* kernel, size_t bytes) {
+  cudaFuncAttributes fa{};
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+  int dev = 0, optin = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+    return e;
+  const size_t most = (size_t)optin - fa.sharedSizeBytes;
+  if (bytes > most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // error helpers -------------------------------------------------------------
 gridff_status set_err(gridff_ctx* ctx, gridff_status st, const char* fmt, ...);
 

@@ -683,7 +683,7 @@ void fused_forward(gridff_mlp* m, const FusedNet& f, const FusedInput& in, int t
   const int per = wide ? 64 : 16;
   const size_t dyn = 2 * (size_t)per * kFusedLd * sizeof(__nv_bfloat16);
   auto fn = wide ? fused_forward_kernel<4> : fused_forward_kernel<1>;
-  if (wide) cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  allow_dyn_smem((const void*)fn, dyn);
   fused_launch(m, fn, (f.Mp + per - 1) / per, 256, dyn, ahead, f, in, train);
 }
 
