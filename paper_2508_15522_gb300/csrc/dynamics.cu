@@ -845,6 +845,7 @@ __device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache&
   // served by that replica's quads alone, against this one (us a call): 4096 x
   // 38 atoms, 200 steps 1073 against 950; 64 x 10 331 against 308; NVE of 1001 x
   // 38 685 against 637.  Two gathers in flight per quad spill (1005).
+  constexpr bool kWide = KIND < 0;      // grids of any size go to the run-time kind (rigid_kind)
   {
     int total = 0;
 #pragma unroll
@@ -853,7 +854,7 @@ __device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache&
       if ((bal >> lane) & 1u) {
         const int slot = k * W + l;
         list[total + __popc(bal & ((1u << lane) - 1u))] =
-            make_int2((int)(unsigned)(((long long)cl[k].ix * g.nyp + cl[k].iy) * g.nzp + cl[k].iz), slot | (sw << 8));
+            refill_entry<kWide>(((long long)cl[k].ix * g.nyp + cl[k].iy) * g.nzp + cl[k].iz, slot, sw);
         sc.key[slot] = key[k];
       }
       total += __popc(bal);
@@ -864,11 +865,11 @@ __device__ __forceinline__ void sw_forces(const GridView& g, const StencilCache&
     for (int j = 0; j < total; j += kQuads) {
       const bool on = j + qd < total;
       const int2 e = list[on ? j + qd : 0];
-      const int s2 = e.y >> 8, slot = e.y & 0xff;
+      const int s2 = refill_sub<kWide>(e), slot = refill_slot(e);
       const int a = __shfl_sync(kFull, ab, s2 * W);      // the entry's template: its replica's
       if (on) {
         float cv[16];
-        gather_runs<KIND>(g, (long long)(unsigned)e.x + qq, __ldg(&par[a + slot]), cv);
+        gather_runs<KIND>(g, refill_record<kWide>(e) + qq, __ldg(&par[a + slot]), cv);
         // runs (a, b) and (a, b + 1), b even, z-node qq go to float4 2p +
         // (qq >> 1) of run pair p = 2a + (b >> 1), half qq & 1: one 8-byte store
         float2* const dst = (float2*)(wval + (size_t)s2 * stride) + 2 * ((qq >> 1) * S + slot) + (qq & 1);
@@ -2154,6 +2155,12 @@ __global__ void fire_reset_kernel(int n, float dt0, float a0, float* dt, float* 
 using SwFn = void (*)(GridView, TemplateView, const int*, int, float*, float*, float*, float*, int*, int*, int*,
                      double*, float*, float*, int*, int, int, int, FireP, Control, int);
 
+// Record kind that picks a sub-warp instance: the instances of one kind index 2^32
+// records, larger grids take the run-time choice (-1), whose list holds 54 bits.
+int rigid_kind(const gridff_grid* grid) {
+  if (!grid) return REC_F32x4;
+  return (unsigned long long)grid->nxp * grid->nyp * grid->nzp <= 1ull << 32 ? grid->kind : -1;
+}
 // Sub-warp rigid kernel for W lanes per replica and R atoms per lane. FP32
 // four-slot grids and 16-bit two-slot grids (FP16 and BF16 share the instance:
 // gather_runs tells them apart) get a build without the other record kinds'
@@ -2363,7 +2370,7 @@ gridff_status enqueue_md_flex(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
 
 gridff_status prepare_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, const LaunchCfg& c,
                             int flags, int* blocks_out) {
-  const KernelShape k = shape_of(R, c, grid ? grid->kind : REC_F32x4);
+  const KernelShape k = shape_of(R, c, R->rigid ? rigid_kind(grid) : grid ? grid->kind : REC_F32x4);
   if (!k.fn) return set_err(ctx, GRIDFF_EINVAL, "launch configuration (kernel %d) does not apply", c.kernel);
   if (c.S < 0 || c.S > GRIDFF_MAX_ATOMS) return set_err(ctx, GRIDFF_EINVAL, "cache slots %d", c.S);
   if (c.kernel == GRIDFF_KERNEL_RIGID_SUBWARP && (flags & GRIDFF_NO_GRID))
@@ -2473,7 +2480,7 @@ gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
               (DevResult*)ctx->result_dev};
   GridView gv = grid ? grid->view() : empty_view();
   const int use_grid = !(flags & GRIDFF_NO_GRID), use_intra = !(flags & GRIDFF_NO_INTRA);
-  const int kind = grid ? grid->kind : REC_F32x4;
+  const int kind = R->rigid ? rigid_kind(grid) : grid ? grid->kind : REC_F32x4;
   const KernelShape k = shape_of(R, c, kind);
   cudaAccessPolicyWindow win{};
   const cudaAccessPolicyWindow* wp = nullptr;
@@ -2731,7 +2738,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
   if (R->rigid) {
     if (!use_grid) return set_err(ctx, GRIDFF_EINVAL, "rigid replicas need the grid term");
     const int W = rigid_subwarp_width(R);
-    const RunSwFn fn = W > 0 ? run_sw_fn(W, sw_rounds(R, W), grid->kind) : nullptr;
+    const RunSwFn fn = W > 0 ? run_sw_fn(W, sw_rounds(R, W), rigid_kind(grid)) : nullptr;
     if (fn) {
       // the sub-warp layout of the relaxation, every atom cached
       const int S = R->max_natoms;
