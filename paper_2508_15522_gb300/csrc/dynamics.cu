@@ -429,7 +429,7 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   // Bonded terms (few per atom): lanes take terms round-robin and add the
   // forces with shared-memory atomics.  Reciprocals come from rsqrtf
   // (1/x = rsqrt(x)^2), not from divisions, except where results are read
-  // (bond_factor()).
+  // (bond_factor(), angle_term(), torsion_term()).
   for (int b = tv.ub_off[t] + lane; b < tv.ub_off[t + 1]; b += 32) {
     const BondTerm B = tv.ub[b];
     const float3 d = sub3(ld3(s_x, B.i), ld3(s_x, B.j));
@@ -442,44 +442,23 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   for (int a = tv.ua_off[t] + lane; a < tv.ua_off[t + 1]; a += 32) {
     const AngleRec A = tv.ua[a];
     const float3 u = sub3(ld3(s_x, A.a), ld3(s_x, A.b)), w = sub3(ld3(s_x, A.c), ld3(s_x, A.b));
-    const float u2 = dot3(u, u), w2 = dot3(w, w), ru = rsqrtf(u2), rw = rsqrtf(w2);
-    const float inv = kReadOut<Acc> ? rsqrtf(u2 * w2) : ru * rw, iu2 = ru * ru, iw2 = rw * rw;
-    const float c = dot3(u, w) * inv;
-    const float dEdc = 2.f * A.k * (c - A.cos0);
-    const float cu = c * iu2, cw = c * iw2;
-    const float3 ga = make_float3(w.x * inv - cu * u.x, w.y * inv - cu * u.y, w.z * inv - cu * u.z);
-    const float3 gc = make_float3(u.x * inv - cw * w.x, u.y * inv - cw * w.y, u.z * inv - cw * w.z);
+    float3 ga, gc;
+    float dEdc;
+    e += angle_term<kReadOut<Acc>>(u, w, A.k, A.cos0, ga, gc, dEdc);
     sh_add3(s_f, A.a, -dEdc * ga.x, -dEdc * ga.y, -dEdc * ga.z);
     sh_add3(s_f, A.c, -dEdc * gc.x, -dEdc * gc.y, -dEdc * gc.z);
     sh_add3(s_f, A.b, dEdc * (ga.x + gc.x), dEdc * (ga.y + gc.y), dEdc * (ga.z + gc.z));
-    e += A.k * (c - A.cos0) * (c - A.cos0);
   }
   for (int k = tv.ut_off[t] + lane; k < tv.ut_off[t + 1]; k += 32) {
     const TorsionRec T = tv.ut[k];
-    const float3 xa = ld3(s_x, T.a), xb = ld3(s_x, T.b), xc = ld3(s_x, T.c), xd = ld3(s_x, T.d);
-    const float3 F = sub3(xa, xb), G = sub3(xb, xc), H = sub3(xd, xc);
-    const float3 A = cross3(F, G), B = cross3(H, G);
-    const float A2 = dot3(A, A), B2 = dot3(B, B), G2 = dot3(G, G);
-    if (A2 < 1e-12f || B2 < 1e-12f || G2 < 1e-12f) continue;   // collinear: no torque
-    const float rA = rsqrtf(A2), rB = rsqrtf(B2), rG = rsqrtf(G2);
-    const float iA2 = rA * rA, iB2 = rB * rB, Gn = G2 * rG;
-    const float iAB = rA * rB;
-    const float cphi = dot3(A, B) * iAB;
-    const float sphi = dot3(cross3(B, A), G) * iAB * rG;
-    float sn, cn;
-    multiple_angle(cphi, sphi, T.n, cn, sn);
-    const float dEdphi = 0.5f * T.V * T.cn0 * T.n * sn;
-    const float FG = dot3(F, G) * iA2 * rG, HG = dot3(H, G) * iB2 * rG;
-    const float ca = -Gn * iA2, cd = Gn * iB2;
-    const float a1 = -ca + FG, b1 = -cd + HG;
-    // gradients of phi with respect to the four atoms, times -dE/dphi
-    const float m0 = -dEdphi * ca, m3 = -dEdphi * cd, m1 = -dEdphi * a1, m2 = -dEdphi * b1;
-    const float h1 = dEdphi * HG, h2 = dEdphi * FG;
-    sh_add3(s_f, T.a, m0 * A.x, m0 * A.y, m0 * A.z);
-    sh_add3(s_f, T.b, m1 * A.x + h1 * B.x, m1 * A.y + h1 * B.y, m1 * A.z + h1 * B.z);
-    sh_add3(s_f, T.c, m2 * B.x + h2 * A.x, m2 * B.y + h2 * A.y, m2 * B.z + h2 * A.z);
-    sh_add3(s_f, T.d, m3 * B.x, m3 * B.y, m3 * B.z);
-    e += 0.5f * T.V * (1.f - T.cn0 * cn);
+    float3 fa, fb, fc, fd;
+    float et;
+    if (!torsion_term<kReadOut<Acc>>(ld3(s_x, T.a), ld3(s_x, T.b), ld3(s_x, T.c), ld3(s_x, T.d), T, fa, fb, fc, fd, et)) continue;
+    e += et;
+    sh_add3(s_f, T.a, fa.x, fa.y, fa.z);
+    sh_add3(s_f, T.b, fb.x, fb.y, fb.z);
+    sh_add3(s_f, T.c, fc.x, fc.y, fc.z);
+    sh_add3(s_f, T.d, fd.x, fd.y, fd.z);
   }
   return enb + (Acc)e;
 }

@@ -218,49 +218,26 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
     if (k < nt) {
       const TorsionRec T = tv.ut[k0 + k];
       const int o = nb + 3 * na + 4 * k;
-      const float3 xa = xyz(s.x[T.a]), xb = xyz(s.x[T.b]), xc = xyz(s.x[T.c]), xd = xyz(s.x[T.d]);
-      const float3 F = sub3(xa, xb), G = sub3(xb, xc), H = sub3(xd, xc);
-      const float3 A = cross3(F, G), B = cross3(H, G);
-      const float A2 = dot3(A, A), B2 = dot3(B, B), G2 = dot3(G, G);
-      if (A2 < 1e-12f || B2 < 1e-12f || G2 < 1e-12f) {   // collinear: no torque
-        for (int c = 0; c < 4; ++c) put3(s.slot, o + c, 0.f, 0.f, 0.f);
-        continue;
-      }
-      const float rA = rsqrtf(A2), rB = rsqrtf(B2), rG = rsqrtf(G2);
-      const float iA2 = rA * rA, iB2 = rB * rB, Gn = G2 * rG;
-      const float iAB = rA * rB;
-      const float cphi = dot3(A, B) * iAB;
-      const float sphi = dot3(cross3(B, A), G) * iAB * rG;
-      float sn, cn;
-      multiple_angle(cphi, sphi, T.n, cn, sn);
-      const float dEdphi = 0.5f * T.V * T.cn0 * T.n * sn;
-      const float FG = dot3(F, G) * iA2 * rG, HG = dot3(H, G) * iB2 * rG;
-      const float ca = -Gn * iA2, cd = Gn * iB2;
-      const float a1 = -ca + FG, b1 = -cd + HG;
-      // gradients of phi with respect to the four atoms, times -dE/dphi
-      const float m0 = -dEdphi * ca, m3 = -dEdphi * cd, m1 = -dEdphi * a1, m2 = -dEdphi * b1;
-      const float h1 = dEdphi * HG, h2 = dEdphi * FG;
-      put3(s.slot, o, m0 * A.x, m0 * A.y, m0 * A.z);
-      put3(s.slot, o + 1, m1 * A.x + h1 * B.x, m1 * A.y + h1 * B.y, m1 * A.z + h1 * B.z);
-      put3(s.slot, o + 2, m2 * B.x + h2 * A.x, m2 * B.y + h2 * A.y, m2 * B.z + h2 * A.z);
-      put3(s.slot, o + 3, m3 * B.x, m3 * B.y, m3 * B.z);
-      e += 0.5f * T.V * (1.f - T.cn0 * cn);
+      float3 fa, fb, fc, fd;
+      float et = 0.f;
+      if (!torsion_term<EX>(xyz(s.x[T.a]), xyz(s.x[T.b]), xyz(s.x[T.c]), xyz(s.x[T.d]), T, fa, fb, fc, fd, et))
+        fa = fb = fc = fd = make_float3(0.f, 0.f, 0.f);
+      e += et;
+      put3(s.slot, o, fa.x, fa.y, fa.z);
+      put3(s.slot, o + 1, fb.x, fb.y, fb.z);
+      put3(s.slot, o + 2, fc.x, fc.y, fc.z);
+      put3(s.slot, o + 3, fd.x, fd.y, fd.z);
     } else if (k < nt + na) {
       const int j = k - nt, o = nb + 3 * j;
       const AngleRec A = tv.ua[a0 + j];
       const float3 xb = xyz(s.x[A.b]);
       const float3 u = sub3(xyz(s.x[A.a]), xb), w = sub3(xyz(s.x[A.c]), xb);
-      const float u2 = dot3(u, u), w2 = dot3(w, w), ru = rsqrtf(u2), rw = rsqrtf(w2);
-      const float inv = EX ? rsqrtf(u2 * w2) : ru * rw, iu2 = ru * ru, iw2 = rw * rw;
-      const float c = dot3(u, w) * inv;
-      const float dEdc = 2.f * A.k * (c - A.cos0);
-      const float cu = c * iu2, cw = c * iw2;
-      const float3 ga = make_float3(w.x * inv - cu * u.x, w.y * inv - cu * u.y, w.z * inv - cu * u.z);
-      const float3 gc = make_float3(u.x * inv - cw * w.x, u.y * inv - cw * w.y, u.z * inv - cw * w.z);
+      float3 ga, gc;
+      float dEdc;
+      e += angle_term<EX>(u, w, A.k, A.cos0, ga, gc, dEdc);
       put3(s.slot, o, -dEdc * ga.x, -dEdc * ga.y, -dEdc * ga.z);
       put3(s.slot, o + 1, dEdc * (ga.x + gc.x), dEdc * (ga.y + gc.y), dEdc * (ga.z + gc.z));
       put3(s.slot, o + 2, -dEdc * gc.x, -dEdc * gc.y, -dEdc * gc.z);
-      e += A.k * (c - A.cos0) * (c - A.cos0);
     } else {
       const int j = k - nt - na;
       const BondTerm B = tv.ub[b0 + j];

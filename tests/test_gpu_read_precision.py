@@ -1,0 +1,73 @@
+"""Precision of the results that are read (evaluations and constant-energy
+dynamics), in both splits of a replica over lanes (a warp; a team of warps):
+no worse than the per-atom pass with its divisions."""
+import numpy as np
+import pytest
+
+from oracle import intra as ointra
+from paper_2508_15522_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+f32 = np.float32
+KE = f32(14.399645)
+ACC = f32(9.648533e-3)
+
+# replicas that go to teams, and to a warp each (more than 8 per SM)
+SPLITS = (200, 1300)
+
+
+@pytest.fixture(scope="module")
+def env():
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2508_15522_gb300 import gridff
+    return gridff, gridff.Context(0)
+
+
+def molecule(n, q=None, mass=None, **terms):
+    """n atoms without nonbonded wells; charges and bonded terms as given (FP32 values)."""
+    m = synth.Molecule(["C"] * n, np.zeros((n, 3)), np.zeros(n) if q is None else q, np.ones(n), np.zeros(n),
+                       np.full(n, 12.0) if mass is None else mass)
+    for k, v in terms.items():
+        setattr(m, k, v)
+    return m
+
+
+@pytest.mark.parametrize("n_rep", SPLITS)
+@pytest.mark.parametrize("term", ["angle", "torsion"])
+def test_bonded_forces_as_the_per_atom_pass(env, term, n_rep):
+    """One angle (torsion) per group of atoms, so that no sums blur it: the median relative
+    error of an atom's force is at most 1.1 times that of the per-atom layout, whose
+    reciprocals are divisions (the same number of roundings; 1.1 for their order)."""
+    G, ctx = env
+    per, k = (3, 42) if term == "angle" else (4, 32)
+    n = per * k
+    idx = np.arange(n, dtype=np.int32).reshape(k, per)
+    g = np.random.default_rng(7)
+    if term == "angle":
+        m = molecule(n, angles=idx, angle_k=np.full(k, 3.0), angle_cos0=np.full(k, -0.25))
+    else:
+        m = molecule(n, torsions=idx, torsion_V=np.full(k, 0.5), torsion_n=np.full(k, 3, np.int32),
+                     torsion_cos_nphi0=np.full(k, -1.0))
+    # bond vectors of 1.1 to 1.6 A in random directions, groups 20 A apart in z
+    step = g.standard_normal((n_rep, k, per, 3))
+    step *= (1.1 + 0.5 * g.random((n_rep, k, per, 1))) / np.linalg.norm(step, axis=-1, keepdims=True)
+    x = np.cumsum(step, 2)
+    x[..., 2] += 20.0 * np.arange(k)[None, :, None]
+    x = x.reshape(n_rep, n, 3).astype(f32)
+    ref = ointra.energy_forces(x[:200].astype(np.float64), m)[1]
+    err = {}
+    for name in ("eval", "per atom"):
+        reps = G.Replicas(ctx, [m], [0] * n_rep)
+        if name == "per atom":
+            reps.set_launch_config(kernel=G.KERNEL_FLEX_QUAD, warps_per_block=4, queue=0)
+        reps.set_state(x.ravel())
+        if name == "eval":
+            F = G.eval(ctx, None, reps, flags=G.NO_GRID)[1]
+        else:
+            G.relax(ctx, None, reps, 1, G.fire_params(f_conv=0.0), flags=G.NO_GRID)
+            F = reps.last_eval()[1]
+        F = F.reshape(n_rep, n, 3)[:200].astype(np.float64)
+        err[name] = np.median(np.linalg.norm(F - ref, axis=-1) / np.linalg.norm(ref, axis=-1))
+    print(term, n_rep, err)
+    assert err["eval"] <= 1.1 * err["per atom"]
