@@ -414,15 +414,15 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
           f[2] += gj.z;
         }
       }
+      if (kReadOut<Acc>) {   // FP64 energies: FP32 sums over one block's partners at most
+        enb += (Acc)e;
+        e = 0.f;
+      }
     }
     if (own) {
       s_f[3 * i] += fi.x;
       s_f[3 * i + 1] += fi.y;
       s_f[3 * i + 2] += fi.z;
-    }
-    if (sizeof(Acc) > sizeof(float)) {   // FP64 energies: FP32 sums over one block's partners at most
-      enb += (Acc)e;
-      e = 0.f;
     }
   }
   __syncwarp();
