@@ -429,7 +429,9 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   // Bonded terms (few per atom): lanes take terms round-robin and add the
   // forces with shared-memory atomics.  Reciprocals come from rsqrtf
   // (1/x = rsqrt(x)^2), not from divisions, except where results are read
-  // (bond_factor(), angle_term(), torsion_term()).
+  // (bond_factor(), angle_term(), torsion_term(); their energies are added in FP64
+  // term by term).
+  Acc sum = enb + (Acc)e;
   for (int b = tv.ub_off[t] + lane; b < tv.ub_off[t + 1]; b += 32) {
     const BondTerm B = tv.ub[b];
     const float3 d = sub3(ld3(s_x, B.i), ld3(s_x, B.j));
@@ -437,14 +439,14 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
     bond_factor<kReadOut<Acc>>(dot3(d, d), B.k, B.r0, c, dr);
     sh_add3(s_f, B.i, c * d.x, c * d.y, c * d.z);
     sh_add3(s_f, B.j, -c * d.x, -c * d.y, -c * d.z);
-    e += B.k * dr * dr;
+    sum += (Acc)(B.k * dr * dr);
   }
   for (int a = tv.ua_off[t] + lane; a < tv.ua_off[t + 1]; a += 32) {
     const AngleRec A = tv.ua[a];
     const float3 u = sub3(ld3(s_x, A.a), ld3(s_x, A.b)), w = sub3(ld3(s_x, A.c), ld3(s_x, A.b));
     float3 ga, gc;
     float dEdc;
-    e += angle_term<kReadOut<Acc>>(u, w, A.k, A.cos0, ga, gc, dEdc);
+    sum += (Acc)angle_term<kReadOut<Acc>>(u, w, A.k, A.cos0, ga, gc, dEdc);
     sh_add3(s_f, A.a, -dEdc * ga.x, -dEdc * ga.y, -dEdc * ga.z);
     sh_add3(s_f, A.c, -dEdc * gc.x, -dEdc * gc.y, -dEdc * gc.z);
     sh_add3(s_f, A.b, dEdc * (ga.x + gc.x), dEdc * (ga.y + gc.y), dEdc * (ga.z + gc.z));
@@ -454,13 +456,13 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
     float3 fa, fb, fc, fd;
     float et;
     if (!torsion_term<kReadOut<Acc>>(ld3(s_x, T.a), ld3(s_x, T.b), ld3(s_x, T.c), ld3(s_x, T.d), T, fa, fb, fc, fd, et)) continue;
-    e += et;
+    sum += (Acc)et;
     sh_add3(s_f, T.a, fa.x, fa.y, fa.z);
     sh_add3(s_f, T.b, fb.x, fb.y, fb.z);
     sh_add3(s_f, T.c, fc.x, fc.y, fc.z);
     sh_add3(s_f, T.d, fd.x, fd.y, fd.z);
   }
-  return enb + (Acc)e;
+  return sum;
 }
 
 // Forces of one flexible replica (positions in s.x) with the grid term by

@@ -209,11 +209,12 @@ __device__ __forceinline__ Acc team_pairs(const TeamState& s, const TemplateView
 // Bonded terms of template t, one per thread of the team: forces on the term's
 // atoms to the term's slots (bonds: the force on atom i; angles: a, b, c;
 // torsions: a, b, c, d).  Returns this thread's share of the energy.
-template <bool EX>
-__device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateView& tv, int t, int tid, int threads) {
+template <class Acc>
+__device__ __forceinline__ Acc team_bonded(const TeamState& s, const TemplateView& tv, int t, int tid, int threads) {
   const int b0 = tv.ub_off[t], a0 = tv.ua_off[t], k0 = tv.ut_off[t];
   const int nb = tv.ub_off[t + 1] - b0, na = tv.ua_off[t + 1] - a0, nt = tv.ut_off[t + 1] - k0;
-  float e = 0.f;
+  constexpr bool EX = kReadOut<Acc>;
+  Acc e = Acc(0);
   for (int k = tid; k < nb + na + nt; k += threads) {
     if (k < nt) {
       const TorsionRec T = tv.ut[k0 + k];
@@ -222,7 +223,7 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
       float et = 0.f;
       if (!torsion_term<EX>(xyz(s.x[T.a]), xyz(s.x[T.b]), xyz(s.x[T.c]), xyz(s.x[T.d]), T, fa, fb, fc, fd, et))
         fa = fb = fc = fd = make_float3(0.f, 0.f, 0.f);
-      e += et;
+      e += (Acc)et;
       put3(s.slot, o, fa.x, fa.y, fa.z);
       put3(s.slot, o + 1, fb.x, fb.y, fb.z);
       put3(s.slot, o + 2, fc.x, fc.y, fc.z);
@@ -234,7 +235,7 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
       const float3 u = sub3(xyz(s.x[A.a]), xb), w = sub3(xyz(s.x[A.c]), xb);
       float3 ga, gc;
       float dEdc;
-      e += angle_term<EX>(u, w, A.k, A.cos0, ga, gc, dEdc);
+      e += (Acc)angle_term<EX>(u, w, A.k, A.cos0, ga, gc, dEdc);
       put3(s.slot, o, -dEdc * ga.x, -dEdc * ga.y, -dEdc * ga.z);
       put3(s.slot, o + 1, dEdc * (ga.x + gc.x), dEdc * (ga.y + gc.y), dEdc * (ga.z + gc.z));
       put3(s.slot, o + 2, -dEdc * gc.x, -dEdc * gc.y, -dEdc * gc.z);
@@ -245,7 +246,7 @@ __device__ __forceinline__ float team_bonded(const TeamState& s, const TemplateV
       float c, dr;
       bond_factor<EX>(dot3(d, d), B.k, B.r0, c, dr);
       put3(s.slot, j, c * d.x, c * d.y, c * d.z);
-      e += B.k * dr * dr;
+      e += (Acc)(B.k * dr * dr);
     }
   }
   return e;
@@ -281,7 +282,7 @@ __device__ __forceinline__ Acc team_forces(const GridView& g, const TemplateView
   float* const fw = s.fw + (size_t)w * 3 * A.N;
   if (A.use_intra) {
     e += team_pairs<NW, Acc>(s, tv, ab, n, lane, w, fw);
-    e += (Acc)team_bonded<kReadOut<Acc>>(s, tv, t, tid, 32 * NW);
+    e += team_bonded<Acc>(s, tv, t, tid, 32 * NW);
   }
   __syncthreads();
   f2 = P = v2 = 0.f;

@@ -94,3 +94,24 @@ def test_bonded_forces_as_the_per_atom_pass(env, term, n_rep):
         err[name] = np.median(np.linalg.norm(F - ref, axis=-1) / np.linalg.norm(ref, axis=-1))
     print(term, n_rep, err)
     assert err["eval"] <= 1.1 * err["per atom"]
+
+
+@pytest.mark.parametrize("n_rep", SPLITS)
+def test_bonded_energies_are_summed_in_fp64(env, n_rep):
+    """600 bonds on a line whose energies are FP32 numbers exactly (odd multiples of 2^-22
+    with 22 bits): their FP64 sum is exact, an FP32 sum of a few is not."""
+    G, ctx = env
+    n, k = 128, 600
+    g = np.random.default_rng(5)
+    pairs = np.array([(i, j) for i in range(n) for j in range(i + 1, n)], np.int32)
+    bonds = pairs[np.sort(g.choice(len(pairs), k, replace=False))]
+    dr = (2 * g.integers(512, 1024, k) + 1) / 2048.0
+    r = (bonds[:, 1] - bonds[:, 0]).astype(float)
+    m = molecule(n, bonds=bonds, bond_k=np.ones(k), bond_r0=r - dr)
+    assert ((r - dr).astype(f32).astype(float) == r - dr).all() and ((dr ** 2).astype(f32).astype(float) == dr ** 2).all()
+    x = np.zeros((n_rep, n, 3), f32)
+    x[:, :, 0] = np.arange(n)
+    reps = G.Replicas(ctx, [m], [0] * n_rep)
+    reps.set_state(x.ravel())
+    E = G.eval(ctx, None, reps, flags=G.NO_GRID)[0]
+    assert (E == (dr ** 2).sum()).all()
