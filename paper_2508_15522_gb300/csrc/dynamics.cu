@@ -1599,13 +1599,14 @@ md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
       s.x[m] = xs[3 * (size_t)off + m];
       s.v[m] = vs[3 * (size_t)off + m];
     }
-    // nonbonded factors {q, alpha log2(e) R (NVE: R), eps} and 1/m or 1/sqrt(m) in the
-    // free fourth slot; zeros up to the next multiple of 32 atoms
+    // nonbonded factors {q, alpha log2(e) R (NVE: R), eps} and, in the free fourth
+    // slot, 1/sqrt(m) (NVE: the half step's dt/2 / m in one division); zeros up to the
+    // next multiple of 32 atoms
     for (int i = lane; i < n; i += 32) {
       float4 p = __ldg(&tv.nb[ab + i]);
       if (!NVE) p.y *= tv.alpha * kLog2e;
       const float mass = __ldg(&tv.body[ab + i]).w;
-      p.w = NVE ? 1.f / mass : rsqrtf(mass);
+      p.w = NVE ? hdt * GRIDFF_ACC / mass : rsqrtf(mass);
       s_nb[i] = p;
     }
     pad_pair_slots(s.x, s_nb, n, lane);
@@ -1636,13 +1637,13 @@ md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
       }
       if (NVE) {
         for (int m = lane; m < 3 * n; m += 32) {
-          const float v = s.v[m] + hdt * GRIDFF_ACC * s_nb[m / 3].w * s.f[m];
+          const float v = s.v[m] + s_nb[m / 3].w * s.f[m];
           s.v[m] = v;
           s.x[m] += dt * v;
         }
         elane = flex_forces_terms<Acc, KIND>(g, use_grid, use_intra, tv, t, ab, n, lane, s, flags, sc, s_nb);
         ++steps_done;
-        for (int m = lane; m < 3 * n; m += 32) s.v[m] += hdt * GRIDFF_ACC * s_nb[m / 3].w * s.f[m];
+        for (int m = lane; m < 3 * n; m += 32) s.v[m] += s_nb[m / 3].w * s.f[m];
         __syncwarp();
         if (trace && rec_every > 0 && (it + 1) % rec_every == 0) {
           const double E = total();

@@ -57,7 +57,7 @@ struct TeamState {
   StencilCache sc;
   float4* x;        // [N] {x, y, z, q}
   float2* nb;       // [N] {alpha log2(e) R, eps} (TEAM_NVE, TEAM_EVAL: {R, eps})
-  float* im;        // [N] 1/m, or 1/sqrt(m) (Langevin)
+  float* im;        // [N] 1/m; 1/sqrt(m) (Langevin); dt/2 / m (NVE)
   float* v;         // [3N]
   float* f;         // [3N] grid force, then the total
   float* fw;        // [NW][3N]
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
       const float* x = A.xs + 3 * ((size_t)off + i);
       s.x[i] = in ? make_float4(x[0], x[1], x[2], p.x) : p;
       s.nb[i] = make_float2(kReadOut<Acc> ? p.y : p.y * (tv.alpha * kLog2e), p.z);
-      s.im[i] = MODE == TEAM_LANGEVIN ? rsqrtf(m) : 1.f / m;
+      s.im[i] = MODE == TEAM_LANGEVIN ? rsqrtf(m) : MODE == TEAM_NVE ? 0.5f * A.dt * GRIDFF_ACC / m : 1.f / m;
       for (int c = 0; c < 3; ++c) s.v[3 * i + c] = in && MODE != TEAM_EVAL ? A.vs[3 * ((size_t)off + i) + c] : 0.f;
     }
     __syncthreads();
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
           }
         }
         for (int i = tid; i < n; i += kThr) {
-          const float h = 0.5f * A.dt * GRIDFF_ACC * s.im[i];
+          const float h = s.im[i];
           float4 x = s.x[i];
           float* xc = &x.x;
 #pragma unroll
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
         __syncthreads();
         ++evals;
         for (int i = tid; i < n; i += kThr) {
-          const float h = 0.5f * A.dt * GRIDFF_ACC * s.im[i];
+          const float h = s.im[i];
           for (int c = 0; c < 3; ++c) s.v[3 * i + c] += h * s.f[3 * i + c];
         }
         if (A.trace && A.rec_every > 0 && (it + 1) % A.rec_every == 0) {

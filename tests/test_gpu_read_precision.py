@@ -1,6 +1,7 @@
 """Precision of the results that are read (evaluations and constant-energy
 dynamics), in both splits of a replica over lanes (a warp; a team of warps):
-no worse than the per-atom pass with its divisions, FP64 sums of the energies."""
+no worse than the per-atom pass with its divisions, FP64 sums of the energies,
+and the velocity update with the mass as divisor."""
 import numpy as np
 import pytest
 
@@ -115,3 +116,22 @@ def test_bonded_energies_are_summed_in_fp64(env, n_rep):
     reps.set_state(x.ravel())
     E = G.eval(ctx, None, reps, flags=G.NO_GRID)[0]
     assert (E == (dr ** 2).sum()).all()
+
+
+@pytest.mark.parametrize("layout", ["team", "warp"])
+def test_velocity_update_divides_by_the_mass(env, layout):
+    """A bond that pulls the atom at x = 0 with exactly 1 eV/A: after one step of 1 fs its
+    coordinate is dt/2 ACC / m rounded once, as FP32 arithmetic gives it."""
+    G, ctx = env
+    masses = (1.0 + 200.0 * np.random.default_rng(9).random(100)).astype(f32)
+    mols = [molecule(2, mass=np.array([m, m], float), bonds=np.array([[0, 1]], np.int32), bond_k=np.ones(1),
+                     bond_r0=np.full(1, 0.5)) for m in masses]
+    reps = G.Replicas(ctx, mols, np.arange(100))
+    if layout == "warp":
+        reps.set_launch_config(kernel=G.KERNEL_FLEX_TERMS)
+    x = np.zeros((100, 2, 3), f32)
+    x[:, 1, 0] = 1.0
+    reps.set_state(x.ravel())
+    G.run(ctx, None, reps, 1, 1.0, flags=G.NO_GRID)
+    got = reps.get_state()[0].reshape(100, 2, 3)[:, 0, 0]
+    assert np.array_equal(got, f32(0.5) * f32(1.0) * ACC / masses)
