@@ -660,8 +660,20 @@ static bool team_fits(const gridff_replicas* R, int NW) {
 //       1216    7.8   5.0  6.0  9.5      10.8   7.0  6.9  11.2      25.1  13.0  12.7  15.4      61.3   65.2  43.8  39.9
 //       2432    9.1   8.6 11.4 18.8      13.0  11.9 13.2  22.2      29.0  25.5  24.1  27.8      74.6  129.3  87.3  79.2
 //       3648   10.9  11.7                15.2  16.4                 34.5  36.5                  97.3  192.9
-// Past W replicas a last round of few replicas costs a whole step latency; up
-// to three rounds it goes to teams (5000 of 22 atoms: 25.0 -> 21.4 us a step).
+// Past W replicas a last round of few replicas costs a whole step latency; where all
+// replicas cost about the same (estimated costs within a tenth) it goes to teams, of
+// molecules of up to 64 atoms also in the second round.  us a step, all on
+// warps / the last round on teams (relaxation; Langevin; NVE):
+//                   W + 304                                   2 W + 304
+//    22 atoms   33.2 / 24.9  34.6 / 26.9  38.1 / 28.5     49.7 / 44.4   53.8 / 48.6   60.0 / 52.1
+//    44..47     56.5 / 48.1  61.5 / 53.4  68.1 / 55.2     89.8 / 85.8   99.8 / 96.8  111.4 / 102.6
+//    64         67.8 / 57.0  74.9 / 63.3  82.6 / 66.3    107.7 / 104.1 119.4 / 117.5 134.5 / 124.8
+//    96          115 / 96.5   122 / 107    138 / 113      179 / 178     199 / 201     222 / 213
+//   113..120     154 / 135    164 / 150    185 / 158      248 / 263     281 / 298     293 / 296
+// and, at one round, 120 atoms with all torsions (three teams an SM) 175 / 151, with W + 608
+// 178 / 170.  In an uneven batch the queue fills the last round's place with the small
+// molecules while the large ones are still at work, and teams only add to that
+// (10..120 atoms, 5000 replicas: 96.9 / 108.6 NVE, 10032: 91.4 / 100.7 relaxation).
 FlexSplit flex_split(const gridff_ctx* ctx, const gridff_replicas* R) {
   const int n = R->max_natoms, n_rep = R->n_rep, W = 32 * ctx->n_sm;
   if (R->cfg.kernel >= 0 || !team_fits(R, 4)) return {0, n_rep};
@@ -671,7 +683,8 @@ FlexSplit flex_split(const gridff_ctx* ctx, const gridff_replicas* R) {
     return {n_rep <= (n > 16 ? W / 4 : W / 8) ? 4 : 2, 0};
   }
   const int rest = n_rep % W;
-  if (n_rep > W && n_rep < 3 * W && rest > 0 && rest <= W / 8) return {4, n_rep - rest};
+  if (n_rep > W && n_rep < (n > 64 ? 2 : 3) * W && rest > 0 && rest <= W / 8 && R->evenness >= 0.9f)
+    return {4, n_rep - rest};
   return {0, n_rep};
 }
 

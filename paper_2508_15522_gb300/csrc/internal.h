@@ -195,6 +195,7 @@ struct gridff_replicas {
   float alpha = 1.5f;
   int max_natoms = 0;
   int max_slots = 0;        // bonded-term slots of the largest template (flexible)
+  float evenness = 1.f;     // estimated cost of the cheapest replica over that of the dearest
   // device
   void* tmpl_blob = nullptr;   // one allocation holding every template array
   TemplateView tv{};

@@ -405,6 +405,7 @@ gridff_status gridff_replicas_create(gridff_ctx* ctx, int32_t n_templates,
   R->alpha = (float)alpha;
   R->max_natoms = max_n;
   R->max_slots = max_slots;
+  R->evenness = (float)(tmpl_cost[rep_tmpl[order.back()]] / tmpl_cost[rep_tmpl[order.front()]]);
   auto bail = [&](gridff_status st, const char* what) {
     gridff_replicas_destroy(R);
     return set_err(ctx, st, "%s", what);

@@ -102,3 +102,31 @@ def test_one_clock_budget(env, batch, call):
         assert st == G.ESTEPLIMIT
     assert 200.0 <= ctx.last_kernel_ms() <= 300.0
     assert ((reps.fire_state()["status"] & G.REP_STEPLIMIT) != 0).all()
+
+
+@pytest.mark.parametrize("sizes, rounds, split", [((22,), 1, True), ((44, 47), 2, True), ((113, 120), 1, True),
+                                                  ((113, 120), 2, False), ((10, 60, 120), 1, False), ((30, 47), 1, False)])
+def test_which_last_rounds_go_to_teams(env, batch, sizes, rounds, split):
+    """Only those of even batches, where a team is faster than the queue: seen by the
+    bits, which differ between the layouts in the order of FP32 sums."""
+    G, ctx, W = env
+    grid = batch[3]
+    sub = synth.rocksalt_slab(ncell=2)
+    mols = [synth.random_flexible_molecule(n, 3, n) for n in sizes]
+    n_rep = rounds * W + 37
+    tof = np.arange(n_rep) % len(mols)
+    pos = [synth.flexible_positions(m, sub, 8, seed=3).astype(np.float32).reshape(8, -1) for m in mols]
+    x = np.concatenate([pos[k][i % 8] for i, k in enumerate(tof)])
+    out = []
+    for default in (True, False):
+        reps = G.Replicas(ctx, mols, tof)
+        if not default:
+            reps.set_launch_config(kernel=G.KERNEL_FLEX_TERMS)
+        reps.set_state(x)
+        G.relax(ctx, grid, reps, 4, G.fire_params(f_conv=0.0))
+        out.append(reps.last_eval()[1])
+        off = reps.atom_offset
+        reps.close()
+    d = np.abs(out[0] - out[1]).max(1)
+    differ = sum(d[off[r]:off[r + 1]].any() for r in range(n_rep))
+    assert differ <= 37 and (differ > 30 if split else differ == 0)
