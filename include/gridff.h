@@ -460,11 +460,13 @@ typedef struct {
 } gridff_launch_config;
 
 /* Fix the launch configuration of relaxations of `reps` (NULL: back to the
- * library's heuristic).  Errors: EINVAL when the configuration does not
- * apply to the replica set (checked here and at launch). */
+ * library's heuristic).  A layout set here serves every replica; the heuristic also
+ * hands small flexible sets, and the last round of even ones, to teams of
+ * 2 to 8 warps per replica, which no layout names.  Errors: EINVAL when the
+ * configuration does not apply to the replica set (checked here and at launch). */
 gridff_status gridff_set_launch_config(gridff_replicas* reps, const gridff_launch_config* cfg);
-/* The configuration gridff_relax would use now (heuristic if none set);
- * use_grid = 0 for relaxations with GRIDFF_NO_GRID. */
+/* The configuration gridff_relax would use now (heuristic if none set: that
+ * of the replicas that teams do not serve); use_grid = 0 for relaxations with GRIDFF_NO_GRID. */
 gridff_status gridff_get_launch_config(const gridff_replicas* reps, int use_grid, gridff_launch_config* cfg);
 
 typedef struct {
@@ -478,8 +480,9 @@ typedef struct {
  * candidate configurations by coordinate descent over the kernel (and warps
  * per block), the stencil staging (cache slots, or the unique-term kernel's
  * global stencil cache), the work queue and the L2
- * window, picks the fastest in atom evaluations per second and makes it the
- * replica set's configuration.  The state (positions, velocities, FIRE
+ * window, and the heuristic itself where it uses teams of warps; picks the
+ * fastest in atom evaluations per second and makes it the replica set's
+ * configuration (if the heuristic won: none set).  The state (positions, velocities, FIRE
  * scalars, status, counters, energies) is restored afterwards.  Allocates
  * scratch for one copy of the state.  trials (may be NULL) receives up to
  * max_trials records; n_trials the number run.

@@ -2678,7 +2678,7 @@ gridff_status gridff_langevin(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
   const double kB = 8.617333262e-5;   // eV/K
   const float kT_acc = (float)(kB * prm->temperature * GRIDFF_ACC);
   GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev0, s));
-  const FlexSplit sp = flex_split(ctx, R);
+  const FlexSplit sp = R->cfg.kernel < 0 ? flex_split(ctx, R) : FlexSplit{0, R->n_rep};
   if (sp.team > 0 && (st = enqueue_team_langevin(ctx, grid, R, sp, nsteps, *prm, (float)c1, (float)c2, kT_acc, flags)) != GRIDFF_OK)
     return st;
   if (sp.n_warp > 0 && (st = enqueue_md_flex<false>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, (float)c1, (float)c2, kT_acc,
@@ -2751,7 +2751,7 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
     run_rigid_kernel<<<blocks, kThreads, dyn, s>>>(gv, R->tv, R->rep_tmpl, R->n_rep, R->x, R->v, R->status,
                                                    R->energy, nsteps, prm->dt, rec_every, dtrace, ctl, S);
   } else {
-    const FlexSplit sp = flex_split(ctx, R);
+    const FlexSplit sp = R->cfg.kernel < 0 ? flex_split(ctx, R) : FlexSplit{0, R->n_rep};
     if (sp.team > 0 && (st = enqueue_team_run(ctx, grid, R, sp, nsteps, *prm, dtrace, flags)) != GRIDFF_OK) return st;
     if (sp.n_warp > 0 && (st = enqueue_md_flex<true>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, 0.f, 0.f, 0.f, 0, 0, rec_every,
                                                      dtrace, prm->clock_budget_s, flags)) != GRIDFF_OK)

@@ -676,7 +676,7 @@ static bool team_fits(const gridff_replicas* R, int NW) {
 // (10..120 atoms, 5000 replicas: 96.9 / 108.6 NVE, 10032: 91.4 / 100.7 relaxation).
 FlexSplit flex_split(const gridff_ctx* ctx, const gridff_replicas* R) {
   const int n = R->max_natoms, n_rep = R->n_rep, W = 32 * ctx->n_sm;
-  if (R->cfg.kernel >= 0 || !team_fits(R, 4)) return {0, n_rep};
+  if (!team_fits(R, 4)) return {0, n_rep};
   if (n_rep <= W / 2) {
     if (team_fits(R, 8) && (n > 96 ? n_rep <= W / 4 : n > 32 && n_rep <= W / 16)) return {8, 0};
     if (n > 32) return n > 96 && n_rep > W / 4 ? FlexSplit{0, n_rep} : FlexSplit{4, 0};

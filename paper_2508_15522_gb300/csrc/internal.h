@@ -270,8 +270,9 @@ gridff_status enqueue_build_poses(gridff_replicas* R, const float* d_poses, int 
 gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_replicas* R, const LaunchCfg& c,
                             int blocks, int nsteps, const gridff_fire_params& P, int flags);
 gridff_status check_fire_params(gridff_ctx* ctx, const gridff_fire_params& P);
-// Flexible batches: the first n_warp replicas of the cost order by the
-// warp-per-replica kernels, the others by teams of `team` warps (flex_team.cu).
+// Flexible batches in the library's own layout (none set): the first n_warp
+// replicas of the cost order by the warp-per-replica kernels, the others by teams
+// of `team` warps (flex_team.cu).
 struct FlexSplit {
   int team;
   int n_warp;

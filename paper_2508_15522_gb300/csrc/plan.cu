@@ -40,7 +40,7 @@ gridff_launch_config to_public(const LaunchCfg& c) {
 
 bool same(const LaunchCfg& a, const LaunchCfg& b) {
   return a.kernel == b.kernel && a.W == b.W && a.wpb == b.wpb && a.S == b.S && a.queue == b.queue &&
-         a.l2win == b.l2win && a.blocks == b.blocks && a.gcache == b.gcache;
+         a.l2win == b.l2win && a.blocks == b.blocks && a.gcache == b.gcache && a.is_default == b.is_default;
 }
 
 // One copy of a replica set's mutable state (tuning trials restore it).
@@ -178,6 +178,12 @@ gridff_status gridff_tune(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
     int blocks = 0;
     gridff_status ps = prepare_relax(ctx, grid, R, c, flags, &blocks);
     if (ps == GRIDFF_OK) {
+      // prepare_relax has loaded the layout's kernel; the team kernels are loaded by
+      // their first launch, which stays out of the time
+      if (c.is_default) {
+        const gridff_status ws = enqueue_relax(ctx, grid, R, c, blocks, 1, P, flags);
+        if (ws != GRIDFF_OK) return ws;
+      }
       GRIDFF_CUDA(ctx, snap(R, snapshot, false, s));
       GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev0, s));
       gridff_status es = enqueue_relax(ctx, grid, R, c, blocks, trial_steps, P, flags);
@@ -204,7 +210,7 @@ gridff_status gridff_tune(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
   };
 
   LaunchCfg best = default_launch_cfg(R, use_grid);
-  best.is_default = false;   // trials are layouts of gridff_launch_config
+  best.is_default = false;   // layouts of gridff_launch_config first
   double best_rate = 0;
   st = trial(best, best_rate);
   for (int pass = 0; pass < 2 && st == GRIDFF_OK; ++pass) {
@@ -262,6 +268,15 @@ gridff_status gridff_tune(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
       }
     }
   }
+  // the heuristic, where it hands replicas to teams, which no layout names
+  if (!R->rigid && st == GRIDFF_OK && flex_split(ctx, R).team > 0) {
+    const LaunchCfg c = default_launch_cfg(R, use_grid);
+    double r = 0;
+    if ((st = trial(c, r)) == GRIDFF_OK && r > best_rate) {
+      best_rate = r;
+      best = c;
+    }
+  }
   cudaError_t e = snap(R, snapshot, false, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (st != GRIDFF_OK) return st;
@@ -270,7 +285,7 @@ gridff_status gridff_tune(gridff_ctx* ctx, const gridff_grid* grid, gridff_repli
   // normalise as the trial did
   for (auto& kv : seen)
     if (kv.second == best_rate) best = kv.first;
-  R->cfg = best;
+  R->cfg = best.is_default ? LaunchCfg() : best;
   if (best_out) *best_out = to_public(best);
   if (n_trials) *n_trials = count;
   return GRIDFF_OK;
