@@ -634,7 +634,7 @@ TeamFn team_fn_m(int mode) {
     case TEAM_RELAX: return flex_team_kernel<NW, KIND, TEAM_RELAX>;
     case TEAM_LANGEVIN: return flex_team_kernel<NW, KIND, TEAM_LANGEVIN>;
     case TEAM_NVE: return flex_team_kernel<NW, KIND, TEAM_NVE>;
-    default: return flex_team_kernel<NW, KIND, TEAM_EVAL>;
+    default: return flex_team_kernel<4, KIND, TEAM_EVAL>;      // eval_team_width
   }
 }
 TeamFn team_fn(int NW, int kind, int mode) {
