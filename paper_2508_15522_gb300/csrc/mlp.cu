@@ -557,7 +557,7 @@ void gemm(cudaStream_t s, const __nv_bfloat16* A, int lda, const __nv_bfloat16* 
 }
 
 // The four-launch form covers the network (a training batch also needs
-// K <= 240 proposals per target: a block evaluates them together).
+// K <= 248 proposals per target: a block evaluates them together).
 bool fused_shape(const gridff_mlp* m) {
   return m->L <= kFusedMaxL && *std::max_element(m->pads.begin(), m->pads.end()) <= kFusedW;
 }
