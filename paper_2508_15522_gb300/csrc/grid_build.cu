@@ -224,9 +224,13 @@ __global__ void radial_table_kernel(int n_f, int n_g, double alpha, double beta,
 // --------------------------------------------------------------------------
 // node values
 // --------------------------------------------------------------------------
-// A warp computes 4 neighbouring columns (consecutive y, one x) x 32
-// consecutive z; warps take these items from a counter, lowest z first (they
-// have the most atoms in range).  Its lanes first test 32 images at a time
+// A warp computes COLS neighbouring columns (consecutive y, one x) x 32
+// consecutive z: 4 columns with the table, 1 without it, where a pair costs about
+// ten times as much.  A warp's first item is fixed, spread over the SMs; the
+// others come from a counter, lowest z first (they have the most atoms in range).
+// A small grid has fewer items than the chip has warps: 75 x 75 x 27 nodes with a
+// cutoff of 25 A, 1425 items of 4 columns from a counter alone, left 63 of 152 SMs
+// without work (14.1 ms, now 2.6).  Its lanes first test 32 images at a time
 // against the item's box and compute the squared in-plane distances to the
 // four columns; then the images that can reach it are taken one by one, their
 // distances broadcast, one lane per z.  Bound by the FP64 pipe: per pair in
@@ -235,7 +239,7 @@ __global__ void radial_table_kernel(int n_f, int n_g, double alpha, double beta,
 // 8 x 8 x 3 rock-salt slab, 113 x 113 x 208 nodes: 12.7 ms (659 ms with a
 // thread per node over every image of every atom and the library functions).
 constexpr int kNodeWarps = 16;
-constexpr int kCols = 4;
+constexpr int kTableCols = 4;
 
 struct NodeTables {
   const double2* tab;          // radial table (TABLE)
@@ -250,7 +254,7 @@ struct NodeTables {
 
 __device__ __forceinline__ double bcast(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-template <bool TABLE>
+template <bool TABLE, int COLS>
 __global__ void __launch_bounds__(32 * kNodeWarps, 1)
 node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double* __restrict__ vals) {
   extern __shared__ __align__(16) double2 s_tab[];
@@ -261,7 +265,7 @@ node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double*
     for (int i = threadIdx.x; i < n; i += blockDim.x) s_tab[i] = nt.tab[i];
     __syncthreads();
   }
-  const int ng = (p.ny + kCols - 1) / kCols, nzc = (p.nz + 31) / 32;
+  const int ng = (p.ny + COLS - 1) / COLS, nzc = (p.nz + 31) / 32;
   const size_t n_nodes = (size_t)p.nx * p.ny * p.nz;
   const double cut2 = fmax(p.morse ? p.rcut2 : 0.0, p.coulomb ? p.ercut2 : 0.0);
   // distances are compared as integers (non-negative doubles order like their
@@ -269,18 +273,16 @@ node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double*
   const unsigned long long rc2 = (unsigned long long)__double_as_longlong(p.morse ? p.rcut2 : 0.0);
   const unsigned long long ec2 = (unsigned long long)__double_as_longlong(p.coulomb ? p.ercut2 : 0.0);
   const int n_k = p.coulomb ? nt.n_k[0] : 0;
-  for (;;) {
-    int item = 0;
-    if (lane == 0) item = atomicAdd(next, 1);
-    item = __shfl_sync(0xffffffffu, item, 0);
+  int item = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (;; item = gridDim.x * kNodeWarps + __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(next, 1) : 0, 0)) {
     if (item >= p.nx * ng * nzc) break;
-    const int zc = item / (p.nx * ng), ix = (item / ng) % p.nx, iy0 = (item % ng) * kCols;
+    const int zc = item / (p.nx * ng), ix = (item / ng) % p.nx, iy0 = (item % ng) * COLS;
     const int iz = zc * 32 + lane;
     const double x = p.x0 + ix * p.dx, z = p.z0 + min(iz, p.nz - 1) * p.dz;
     const double zlo = p.z0 + zc * 32 * p.dz, zhi = p.z0 + min(zc * 32 + 31, p.nz - 1) * p.dz;
-    double y[kCols], vP[kCols], vL[kCols], phi[kCols];
+    double y[COLS], vP[COLS], vL[COLS], phi[COLS];
 #pragma unroll
-    for (int c = 0; c < kCols; ++c) {
+    for (int c = 0; c < COLS; ++c) {
       y[c] = p.y0 + (iy0 + c) * p.dy;      // columns past ny are computed and not stored
       vP[c] = vL[c] = phi[c] = 0.0;
     }
@@ -288,14 +290,14 @@ node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double*
     bool have = false;
     for (int j0 = 0; j0 < nt.n_img; j0 += 32) {
       const int j = j0 + lane;
-      double rho2[kCols];
+      double rho2[COLS];
       bool near = false;
       if (j < nt.n_img) {
         const SubImage* im = nt.img + j;
         const double ddx = x - im->x, yj = im->y, zj = im->z;
         double least = 1e300;
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) {
+        for (int c = 0; c < COLS; ++c) {
           const double ddy = y[c] - yj;
           rho2[c] = ddx * ddx + ddy * ddy;
           least = fmin(least, rho2[c]);
@@ -315,11 +317,11 @@ node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double*
           z_prev = zj;
           have = true;
         }
-        double u[kCols];
+        double u[COLS];
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) u[c] = bcast(rho2[c], src) + dz2;
+        for (int c = 0; c < COLS; ++c) u[c] = bcast(rho2[c], src) + dz2;
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) {
+        for (int c = 0; c < COLS; ++c) {
           const unsigned long long ub = (unsigned long long)__double_as_longlong(u[c]);
           if (ub >= rc2 && ub >= ec2) continue;
           const int hi = (int)(ub >> 32), idx = tab_index(hi);
@@ -354,22 +356,22 @@ node_values_kernel(BuildParams p, NodeTables nt, int* __restrict__ next, double*
     // reciprocal part: lanes compute the phases e^{i k.rho} of 32 vectors,
     // then every vector's G(z) is added with the broadcast phases
     for (int k0 = 0; k0 < n_k; k0 += 32) {
-      double pc[kCols], ps[kCols];
+      double pc[COLS], ps[COLS];
       if (k0 + lane < n_k) {
         const double2 kv = nt.kvec[nt.k_list[k0 + lane]];
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) sincos(kv.x * x + kv.y * y[c], &ps[c], &pc[c]);
+        for (int c = 0; c < COLS; ++c) sincos(kv.x * x + kv.y * y[c], &ps[c], &pc[c]);
       }
       const int cnt = min(32, n_k - k0);
       for (int t = 0; t < cnt; ++t) {
         const double2 g = nt.G[(size_t)(k0 + t) * p.nz + min(iz, p.nz - 1)];
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) phi[c] += g.x * bcast(pc[c], t) - g.y * bcast(ps[c], t);
+        for (int c = 0; c < COLS; ++c) phi[c] += g.x * bcast(pc[c], t) - g.y * bcast(ps[c], t);
       }
     }
     if (iz < p.nz) {
 #pragma unroll
-      for (int c = 0; c < kCols; ++c) {
+      for (int c = 0; c < COLS; ++c) {
         if (iy0 + c >= p.ny) break;
         const size_t node = ((size_t)ix * p.ny + iy0 + c) * p.nz + iz;
         if (p.coulomb) vals[(size_t)p.slotC * n_nodes + node] = kKe * (phi[c] + p.bg + p.dip * z);
@@ -1026,17 +1028,16 @@ gridff_status gridff_build_grid(gridff_ctx* ctx, const gridff_substrate* sub,
   nt.n_g = p.coulomb ? intervals(p.ercut2) : 1;
   const size_t tab_bytes = ((kFCoef / 2) * (size_t)nt.n_f + (kGCoef / 2) * (size_t)nt.n_g) * sizeof(double2);
   const bool table = alpha * rcut <= 30.0 && s_tol <= 6.0 && a_R <= 100.0 && tab_bytes <= 200 * 1024;
-  const void* fn = table ? (const void*)node_values_kernel<true> : (const void*)node_values_kernel<false>;
-  if (table) {
+    if (table) {
     double2* d_tab = nullptr;
     if (df.alloc(&d_tab, tab_bytes) != cudaSuccess) return bail(set_err(ctx, GRIDFF_ENOMEM, "radial table"));
     radial_table_kernel<<<(std::max(nt.n_f, nt.n_g) + 63) / 64, 64, 0, s>>>(nt.n_f, nt.n_g, alpha, beta, d_tab);
     nt.tab = d_tab;
-    if (allow_dyn_smem(fn, tab_bytes) != cudaSuccess)
+    if (allow_dyn_smem((const void*)node_values_kernel<true, kTableCols>, tab_bytes) != cudaSuccess)
       return bail(set_err(ctx, GRIDFF_ECUDA, "radial table of %zu bytes", tab_bytes));
-    node_values_kernel<true><<<ctx->n_sm, 32 * kNodeWarps, tab_bytes, s>>>(p, nt, d_next, vals);
+    node_values_kernel<true, kTableCols><<<ctx->n_sm, 32 * kNodeWarps, tab_bytes, s>>>(p, nt, d_next, vals);
   } else {
-    node_values_kernel<false><<<ctx->n_sm, 32 * kNodeWarps, 0, s>>>(p, nt, d_next, vals);
+    node_values_kernel<false, 1><<<ctx->n_sm, 32 * kNodeWarps, 0, s>>>(p, nt, d_next, vals);
   }
   if (cudaGetLastError() != cudaSuccess) return bail(set_err(ctx, GRIDFF_ECUDA, "node kernel launch"));
   if (opts->keep_f64) {
