@@ -407,8 +407,11 @@ gridff_status gridff_template_factors(const gridff_replicas* reps, int32_t t, fl
  * Rigid replicas apply the rule to (COM velocity, total force) and (body
  * angular velocity, body torque).  Without GRIDFF_CONTINUE the FIRE
  * scalars and status are reset first.  result may be NULL.  The result
- * does not depend on the layout or schedule beyond FP32 summation order
- * (rigid layouts: bit for bit).
+ * does not depend on the layout or schedule beyond FP32 summation order.
+ * Rigid replicas: bit for bit the same at equal kernel and lanes_per_replica,
+ * whatever the schedule, block cap and other replicas of the set; the heuristic
+ * takes the lanes from the molecule's and the set's size (gridff_launch_config
+ * fixes them).
  * Errors: EINVAL, ECUDA, EABORTED, ESTEPLIMIT (state is consistent),
  * ETIMEOUT (rigid sub-warp layout: a later part of a relaxation cut into parts
  * gave up waiting for the parts before it; the replicas concerned keep the state of

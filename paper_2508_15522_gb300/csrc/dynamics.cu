@@ -276,13 +276,6 @@ __device__ __forceinline__ Acc flex_forces(const GridView& g, bool use_grid, boo
   return e;
 }
 
-// Intramolecular forces of one flexible replica, each term evaluated once:
-// the lanes split the terms and add every term's forces to its atoms in
-// s_f (nonbonded pairs in the registers of the atoms' owner lanes, the
-// reactions passed by shuffles; bonded terms with atomics).  Returns this
-// lane's share of the energy.  Same terms as
-// intra_quad (reduced UFF-like form; nonbonded on pairs more than two bonds
-// apart), without the per-atom repetition.
 // Nonbonded force factor c (F_i = c d, d = x_i - x_j) and energy of one pair
 // (Morse with mixed R_i + R_j and eps_i eps_j, plus Coulomb), from per-atom
 // factors prepared once per replica: pi = {k_e q_i, a R_i, eps_i, -} for
@@ -358,6 +351,13 @@ __device__ __forceinline__ float3 nb_steps(const float* s_x, const float4* s_nb,
   return g;
 }
 
+// Intramolecular forces of one flexible replica, each term evaluated once:
+// the lanes split the terms and add every term's forces to its atoms in
+// s_f (nonbonded pairs in the registers of the atoms' owner lanes, the
+// reactions passed by shuffles; bonded terms with atomics).  Returns this
+// lane's share of the energy.  Same terms as
+// intra_quad (reduced UFF-like form; nonbonded on pairs more than two bonds
+// apart), without the per-atom repetition.
 template <class Acc>
 __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float* s_x, float* s_f, const float4* s_nb) {
   Acc enb = Acc(0);
