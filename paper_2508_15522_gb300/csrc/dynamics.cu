@@ -2423,11 +2423,18 @@ cudaError_t launch_ex(void (*fn)(KArgs...), int blocks, int threads, size_t dyn,
 // Parts per task of the rigid queue.  Whole tasks leave warps idle in the last
 // round (4096 replicas of 38 atoms: 2048 tasks on 1216 warps take 2 rounds for
 // 1.68 of work); with C parts per task the rounds are ceil(C tasks / warps) / C.
-// A part costs about one and a half iterations more (its state through L2, every
-// stencil of its atoms refilled), so C minimises the sum.  Parts are at most 4096
+// A part costs some iterations more (its state through L2, every stencil of its
+// atoms refilled), 3.5 of them here, so C minimises the sum.  Parts are at most 4096
 // iterations (0.2 s of the largest molecules): the bounded wait counts anew with
-// every part that ends.
-// 4096 x 38 atoms, 200 iterations a call: 1189 -> 1073 us (4 parts).
+// every part that ends.  us of 200 iterations by C (and iterations a part costs, from
+// C = 4 to 12):
+//                            C = 1     2     3     4     5     6     8    12
+//   10 atoms, 12000 replicas  1037   918   926   940   934   965   981  1022   (2.0)
+//   24,        6000            969   784   737   721   733   743   768   824   (3.6)
+//   38,        4096            932   865   869   853   840   859   873   926   (2.2)
+//   38,       20000           3807  3775  3816  3867  3916  3973  4090  4347   (3.2)
+//   60,        1600            721   572   535   552   550   553   564   595   (1.5)
+//  120,        1300           1216  1046   998   986   991  1000  1036  1110   (3.0)
 static int sw_queue_parts(long long tasks, long long warps, int nsteps) {
   if (tasks <= warps) return 1;
   const int least = std::max(2, (nsteps + 4095) / 4096);
@@ -2435,7 +2442,7 @@ static int sw_queue_parts(long long tasks, long long warps, int nsteps) {
   int best = 1;
   double best_cost = (double)((tasks + warps - 1) / warps) * nsteps;
   for (int C = least; C <= most && nsteps / C >= 32; ++C) {
-    const double cost = (double)((tasks * C + warps - 1) / warps) / C * (nsteps + 1.5 * C);
+    const double cost = (double)((tasks * C + warps - 1) / warps) / C * (nsteps + 3.5 * C);
     if (cost < best_cost * (1 - 1e-9)) {
       best_cost = cost;
       best = C;
