@@ -453,14 +453,10 @@ __device__ Acc intra_terms(const TemplateView& tv, int t, int lane, const float*
   }
   for (int k = tv.ut_off[t] + lane; k < tv.ut_off[t + 1]; k += 32) {
     const TorsionRec T = tv.ut[k];
-    float3 fa, fb, fc, fd;
-    float et;
-    if (!torsion_term<kReadOut<Acc>>(ld3(s_x, T.a), ld3(s_x, T.b), ld3(s_x, T.c), ld3(s_x, T.d), T, fa, fb, fc, fd, et)) continue;
-    sum += (Acc)et;
-    sh_add3(s_f, T.a, fa.x, fa.y, fa.z);
-    sh_add3(s_f, T.b, fb.x, fb.y, fb.z);
-    sh_add3(s_f, T.c, fc.x, fc.y, fc.z);
-    sh_add3(s_f, T.d, fd.x, fd.y, fd.z);
+    torsion_term<kReadOut<Acc>, false>(
+        ld3(s_x, T.a), ld3(s_x, T.b), ld3(s_x, T.c), ld3(s_x, T.d), T, sum, [&](int i, float x, float y, float z) {
+          sh_add3(s_f, i == 0 ? T.a : i == 1 ? T.b : i == 2 ? T.c : T.d, x, y, z);
+        });
   }
   return sum;
 }
@@ -1429,7 +1425,7 @@ relax_flex_terms_kernel(GridView g, TemplateView tv, const int* __restrict__ rep
   float4* s_nb = (float4*)(wbase + cache_bytes(S));
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
-  const unsigned long long t0 = lane == 0 ? budget_start(ctl) : 0;
+  const unsigned long long t0 = gtimer();
   for (int k = warp;; k += n_warps) {
     if (order) {
       int next = 0;
@@ -1575,7 +1571,7 @@ md_flex_kernel(GridView g, TemplateView tv, const int* __restrict__ rep_tmpl,
   float4* s_nb = (float4*)(wbase + cache_bytes(S));
   const int warp = blockIdx.x * WPB + wib;
   const int n_warps = gridDim.x * WPB;
-  const unsigned long long t0 = lane == 0 ? budget_start(ctl) : 0;
+  const unsigned long long t0 = gtimer();
   const float hdt = 0.5f * dt;
   const float sq_kT = sqrtf(kT_acc);
   for (int k = warp;; k += n_warps) {
@@ -2296,6 +2292,15 @@ static gridff_status ensure_gcache(gridff_ctx* ctx, gridff_replicas* R) {
   return GRIDFF_OK;
 }
 
+// A split call (warp kernel, then team kernel) with a clock budget: its start, for
+// the second kernel.  The warp kernels count from their own start: a shared one cost
+// the relaxation of 16384 uneven replicas 0.4 to 0.8 % (2540 us), by its registers.
+__global__ void mark_start_kernel(DevResult* res) { res->t0 = gtimer(); }
+static void mark_start(gridff_ctx* ctx, FlexSplit sp, double budget_s) {
+  if (sp.team > 0 && sp.n_warp > 0 && budget_s > 0)
+    mark_start_kernel<<<1, 1, 0, ctx->stream>>>((DevResult*)ctx->result_dev);   // errors: at the next launch's check
+}
+
 using MdFlexFn = void (*)(GridView, TemplateView, const int*, const int*, const int*, int, float*, float*, int*, double*,
                           int, float, float, float, float, unsigned long long, long long, int, double*, int, Control, int,
                           int, int, float4*, int*);
@@ -2513,14 +2518,15 @@ gridff_status enqueue_relax(gridff_ctx* ctx, const gridff_grid* grid, gridff_rep
       break;
     case GRIDFF_KERNEL_FLEX_TERMS: {
       const int* ord = c.queue ? (const int*)R->order : nullptr;
-      if (sp.team > 0) {
-        const gridff_status ts = enqueue_team_relax(ctx, grid, R, sp, nsteps, P, flags);
-        if (ts != GRIDFF_OK) return ts;
-      }
+      mark_start(ctx, sp, P.clock_budget_s);
       if (sp.n_warp > 0) e = launch_ex(flex_terms_fn(c.wpb, kind, c.gcache != 0), blocks, k.threads, k.dyn, s, wp, gv, R->tv,
                     (const int*)R->rep_tmpl, (const int*)R->rep_off, ord, sp.n_warp, R->x, R->v, R->fire_dt,
                     R->fire_alpha, R->fire_nplus, R->status, R->steps, R->energy, R->last_x, R->last_f, nsteps, fp,
                     ctl, use_grid, use_intra, c.S, R->gval, R->gkey);
+      if (sp.team > 0 && e == cudaSuccess) {
+        const gridff_status ts = enqueue_team_relax(ctx, grid, R, sp, nsteps, P, flags);
+        if (ts != GRIDFF_OK) return ts;
+      }
       break;
     }
     default:
@@ -2686,10 +2692,11 @@ gridff_status gridff_langevin(gridff_ctx* ctx, const gridff_grid* grid, gridff_r
   const float kT_acc = (float)(kB * prm->temperature * GRIDFF_ACC);
   GRIDFF_CUDA(ctx, cudaEventRecord(ctx->ev0, s));
   const FlexSplit sp = R->cfg.kernel < 0 ? flex_split(ctx, R) : FlexSplit{0, R->n_rep};
-  if (sp.team > 0 && (st = enqueue_team_langevin(ctx, grid, R, sp, nsteps, *prm, (float)c1, (float)c2, kT_acc, flags)) != GRIDFF_OK)
-    return st;
+  mark_start(ctx, sp, prm->clock_budget_s);
   if (sp.n_warp > 0 && (st = enqueue_md_flex<false>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, (float)c1, (float)c2, kT_acc,
                                                     prm->seed, prm->step0, 0, nullptr, prm->clock_budget_s, flags)) != GRIDFF_OK)
+    return st;
+  if (sp.team > 0 && (st = enqueue_team_langevin(ctx, grid, R, sp, nsteps, *prm, (float)c1, (float)c2, kT_acc, flags)) != GRIDFF_OK)
     return st;
   DevResult h{};
   return finish_launch(ctx, &h);
@@ -2759,10 +2766,11 @@ gridff_status gridff_run(gridff_ctx* ctx, const gridff_grid* grid, gridff_replic
                                                    R->energy, nsteps, prm->dt, rec_every, dtrace, ctl, S);
   } else {
     const FlexSplit sp = R->cfg.kernel < 0 ? flex_split(ctx, R) : FlexSplit{0, R->n_rep};
-    if (sp.team > 0 && (st = enqueue_team_run(ctx, grid, R, sp, nsteps, *prm, dtrace, flags)) != GRIDFF_OK) return st;
+    mark_start(ctx, sp, prm->clock_budget_s);
     if (sp.n_warp > 0 && (st = enqueue_md_flex<true>(ctx, grid, R, sp.n_warp, nsteps, prm->dt, 0.f, 0.f, 0.f, 0, 0, rec_every,
                                                      dtrace, prm->clock_budget_s, flags)) != GRIDFF_OK)
       return st;
+    if (sp.team > 0 && (st = enqueue_team_run(ctx, grid, R, sp, nsteps, *prm, dtrace, flags)) != GRIDFF_OK) return st;
   }
   DevResult h{};
   gridff_status rs = finish_launch(ctx, &h);

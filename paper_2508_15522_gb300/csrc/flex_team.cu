@@ -219,15 +219,8 @@ __device__ __forceinline__ Acc team_bonded(const TeamState& s, const TemplateVie
     if (k < nt) {
       const TorsionRec T = tv.ut[k0 + k];
       const int o = nb + 3 * na + 4 * k;
-      float3 fa, fb, fc, fd;
-      float et = 0.f;
-      if (!torsion_term<EX>(xyz(s.x[T.a]), xyz(s.x[T.b]), xyz(s.x[T.c]), xyz(s.x[T.d]), T, fa, fb, fc, fd, et))
-        fa = fb = fc = fd = make_float3(0.f, 0.f, 0.f);
-      e += (Acc)et;
-      put3(s.slot, o, fa.x, fa.y, fa.z);
-      put3(s.slot, o + 1, fb.x, fb.y, fb.z);
-      put3(s.slot, o + 2, fc.x, fc.y, fc.z);
-      put3(s.slot, o + 3, fd.x, fd.y, fd.z);
+      torsion_term<EX, true>(xyz(s.x[T.a]), xyz(s.x[T.b]), xyz(s.x[T.c]), xyz(s.x[T.d]), T, e,
+                             [&](int i, float x, float y, float z) { put3(s.slot, o + i, x, y, z); });
     } else if (k < nt + na) {
       const int j = k - nt, o = nb + 3 * j;
       const AngleRec A = tv.ua[a0 + j];
@@ -367,15 +360,9 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) flex_team_kernel(GridView g,
   constexpr int kThr = 32 * NW;
   const int tid = threadIdx.x;
   TeamState s = team_state(dyn_smem, NW, A.N, A.S, A.n_slots);
-  const unsigned long long t0 = MODE != TEAM_EVAL && tid == 0 ? budget_start(ctl) : 0;
   // stop bits every 32 steps (abort flag, clock budget), the same in every thread
   auto stop = [&]() {
-    if (tid == 0) {
-      int b = 0;
-      if (*ctl.abort_flag) b |= GRIDFF_REP_ABORTED;
-      if (ctl.budget_ns && gtimer() - t0 > ctl.budget_ns) b |= GRIDFF_REP_STEPLIMIT;
-      *s.word = b;
-    }
+    if (tid == 0) *s.word = call_stop_bits(ctl);
     __syncthreads();
     const int b = *s.word;
     __syncthreads();

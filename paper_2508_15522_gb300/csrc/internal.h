@@ -169,7 +169,7 @@ struct DevResult {
   int next;           // work-queue position (replicas handed out so far)
   int handoff_timeouts;   // parts of split relaxations that did not receive the one before in time
   int team_next;      // the same of the team kernel: both run in a call whose batch is split
-  unsigned long long t0;   // global timer at the start of the call's first kernel (flexible, with a clock budget)
+  unsigned long long t0;   // global timer at the call's start (team kernel with a clock budget)
 };
 
 // Launch configuration of a relaxation (mirrors gridff_launch_config).
