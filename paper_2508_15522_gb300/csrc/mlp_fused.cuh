@@ -111,7 +111,7 @@ __device__ __forceinline__ uint4 load_weights(const uint4* p) {
 // fragment-ordered operand B, k = 0 .. 32 kp - 1.  The whole share of a layer (up
 // to 128 registers) is requested at once and one layer ahead: the weights come
 // from L2, and a load per step of 32 left the kernels waiting (forward 27 us,
-// backward 34 us at 2048 rows, now 14 and 20).
+// backward 34 us at 2048 rows, now 15 and 15).
 struct RowsB {
   uint4 v[4][kFusedW / 32];
 };

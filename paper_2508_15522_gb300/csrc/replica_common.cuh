@@ -279,8 +279,9 @@ constexpr float kLog2e = 1.44269504088896341f;   // log2(e)
 // factors prepared, b = alpha log2(e) R, and one ex2 (rounding 3e-7 of the
 // exponential); evaluations and constant-energy dynamics, which are read as
 // results, the difference in FP32 and expf, b = R.  Either way an evaluation of
-// 4097 uneven molecules takes 106 us and constant-energy dynamics of 1024 x 47
-// atoms 26 us a step: neither is bound by the pairs' instructions.
+// 4097 uneven molecules took 106 us (117 with the divisions and FP64 sums below) and
+// constant-energy dynamics of 1024 x 47 atoms takes 27 us a step: neither is bound by the
+// pairs' instructions.
 template <class Acc>
 constexpr bool kReadOut = sizeof(Acc) > sizeof(float);
 template <bool EX>
@@ -292,7 +293,7 @@ __device__ __forceinline__ float pair_exp(float alpha, float a, float r, float b
 // of zero length has no direction and no force.  EX as above, with the length by
 // sqrtf: r2 rsqrt(r2) is two roundings worse, which a stiff bond turns into most
 // of an evaluation's error (relative, of 4097 uneven molecules: 1.3e-6, with sqrtf 1.1e-6,
-// in 106 us either way).
+// in the same time).
 template <bool EX>
 __device__ __forceinline__ void bond_factor(float r2, float k, float r0, float& c, float& dr) {
   if (EX) {
